@@ -24,7 +24,7 @@ template <class L> int launch_sweep_h16(int, const SweepArgs&, const void*, int,
 template <class L> int occupancy_h16(int, int*, int*);
 template <class L>
 int launch_stencil(const double*, double*, const double*, const Coefs<double>&, int64_t, int, int,
-                   int, int, int, double*, int, void*, const int*);
+                   int, int, int, double*, int, int, void*, const int*);
 }  // namespace pkr
 
 #define PKR_CK(call)                                     \
@@ -202,6 +202,7 @@ struct pkr_plan {
     double* host;   // pinned: [0] mean, [1..4] residual, [5] import mean, [6] flag (int),
                     // [7] binary16 overflow flag (int)
     bool stencil;          // omega = 1, binary64: the state is Phi alone (scalar stencil)
+    int planes;            // stencil mode: z chunk of the plane form, 0: one thread per site
     double* Ps[2];         // stencil mode: Phi ping-pong
     double* St;            // stencil mode: sum_i chi_i S(x - v_i)
     Coefs<double> cchi;    // stencil mode: chi_c in the weight slot (builds St)
@@ -247,7 +248,7 @@ int launch_stencil_step(pkr_plan* P, const double* in, double* out, const double
     const int nx = (int)n[0], ny = (int)n[1], nz = (int)n[2];
     int rc = 0;
 #define PKR_ST(LL) launch_stencil<LL>(in, out, add, c, P->V, nx, ny, nz, P->small, check, \
-                                      P->partials, P->grid, P->stream, P->stop_arg)
+                                      P->partials, P->grid, P->planes, P->stream, P->stop_arg)
     switch (P->prob.lattice) {
     case PKR_D1Q5: rc = PKR_ST(D1Q5); break;
     case PKR_D1Q9: rc = PKR_ST(D1Q9); break;
@@ -476,6 +477,39 @@ int capture_steps(pkr_plan* P, double tol, int tol_kind)
     return PKR_OK;
 }
 
+// Form and grid of the scalar stencil.  3D sets on grids that give every SM
+// a plane tile take the plane form, in chunks of z: the chunk length with the
+// least work on the busiest SM, a chunk costing its planes and about four
+// more for the 2 R partial ones around it (256^3: seven chunks of 37 planes,
+// 1.69 ms a step; five of 52, the fewest with four blocks per SM, 1.88 ms).
+// Other grids take one thread per site.
+void stencil_geometry(pkr_plan* P)
+{
+    const int64_t* n = P->prob.n;
+    P->planes = 0;
+    if (P->lat.dim == 3 && !P->small) {
+        const int64_t tiles = ((n[0] + 31) / 32) * ((n[1] + 15) / 16);
+        int64_t best = 0, items = 0;
+        for (int64_t cz = n[2]; cz >= 6 || cz == n[2]; --cz) {
+            const int64_t it = tiles * ((n[2] + cz - 1) / cz);
+            const int64_t cost = ((it + P->nsm - 1) / P->nsm) * (cz + 4);
+            if (it >= P->nsm && (best == 0 || cost < best)) {
+                best = cost;
+                items = it;
+                P->planes = (int)cz;
+            }
+        }
+        if (P->planes > 0) {
+            P->grid = (int)(items < kMaxGridBlocks ? items : kMaxGridBlocks);
+            return;
+        }
+    }
+    const int tb = stencil_block(P->V, P->nsm);
+    int64_t g = (P->V + tb - 1) / tb;
+    if (g > (int64_t)P->nsm * 8) g = (int64_t)P->nsm * 8;
+    P->grid = (int)g;
+}
+
 size_t plan_bytes(const pkr_problem* p, const LatticeInfo& li, int64_t V, int grid_max)
 {
     const size_t e = (size_t)elem_bytes(p->precision);
@@ -625,10 +659,7 @@ int plan_create(const pkr_problem* p, void* stream, pkr_plan** out, bool spare)
         return PKR_EINVAL;
     }
     if (P->stencil) {
-        const int tb = stencil_block(P->V, nsm);
-        int64_t g = (P->V + tb - 1) / tb;
-        if (g > (int64_t)nsm * 8) g = (int64_t)nsm * 8;
-        P->grid = (int)g;
+        stencil_geometry(P);
         P->variant = 0;
     } else if (set_variant(P, var) != PKR_OK) {
         delete P;
