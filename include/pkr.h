@@ -231,10 +231,13 @@ int pkr_plan_load_source(pkr_plan *plan, const double *rho, int rho_on_host);
  * drops below tol (tol <= 0: never).  stats may be NULL.  Returns PKR_OK,
  * PKR_EDIVERGED or PKR_ECUDA.  Synchronises once per check; except that a
  * binary64 run that checks every step (check_every = 1, tol > 0, steps >= 64)
- * runs its steps as a CUDA graph of 64 steps captured on a stream of the plan
- * and launched on the plan's stream, with the stopping rule applied on the
- * device after each check: same steps and stopping step, one synchronisation
- * per 64 steps. */
+ * applies the stopping rule on the device: same steps and stopping step.  On
+ * small grids (a few 32-site tiles per SM; variant -1) its steps run in
+ * cooperative launches of up to 8192 steps, synchronising once per launch;
+ * the population sweep then steps through a third array, allocated at the
+ * first such run.  On other grids they run as a CUDA graph of 64 steps
+ * captured on a stream of the plan and launched on the plan's stream, one
+ * synchronisation per 64 steps. */
 int pkr_plan_run(pkr_plan *plan, int64_t steps, double tol, int tol_kind, int check_every,
                  pkr_stats *stats);
 

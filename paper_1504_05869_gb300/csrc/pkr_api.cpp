@@ -25,6 +25,8 @@ template <class L> int occupancy_h16(int, int*, int*);
 template <class L>
 int launch_stencil(const double*, double*, const double*, const Coefs<double>&, int64_t, int, int,
                    int, int, int, double*, int, int, void*, const int*);
+template <class L> int resident_form(int64_t, int, int, int);
+template <class L> int launch_resident(int, const CoopArgs&, const Coefs<double>&, void*);
 }  // namespace pkr
 
 #define PKR_CK(call)                                     \
@@ -224,6 +226,10 @@ struct pkr_plan {
                            // index of the step being captured
     double gtol;           // tolerance it was captured for
     const int* stop_arg;   // &ctl->stop while capturing, else nullptr
+    // resident runs (pkr_resident.cuh): form (-1: not looked up yet) and, for
+    // the population form, the third array it steps through
+    int resident;
+    void* pop3;
     bool loaded;
     Coefs<double> c64;
     Coefs<float> c32;
@@ -418,6 +424,121 @@ constexpr int kStallChecks = 4;
 // arrays are back at the same parity after a full replay).
 constexpr int kGraphSteps = 64;
 
+// Device and host copies of the rule's state; the step barrier's counter
+// follows the device one.
+constexpr size_t kCtlBytes = 128;
+int alloc_ctl(pkr_plan* P)
+{
+    static_assert(sizeof(RunCtl) <= 64, "the counter sits at byte 64");
+    if (cudaMalloc((void**)&P->ctl, kCtlBytes) != cudaSuccess ||
+        cudaMallocHost((void**)&P->hctl, sizeof(RunCtl)) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(P->ctl);
+        P->ctl = nullptr;
+        return PKR_ENOMEM;
+    }
+    return PKR_OK;
+}
+
+// Steps per launch of a resident run: tens of milliseconds at most.
+constexpr int64_t kResidentSteps = 8192;
+
+// Form of a resident run of this plan (0: none).  Only where the plan's
+// one-step kernel computes the same values: the per-site stencil, or the
+// library's own choice of sweep geometry.  Tiles: 4 per SM for the stencil,
+// 2 per SM for the sweep (8 + 1 warps of a tile each).
+int resident_of(pkr_plan* P)
+{
+    if (P->resident >= 0) return P->resident;
+    P->resident = 0;
+    if (P->prob.precision != PKR_FP64 || P->prob.variant >= 0 || (P->stencil && P->planes > 0))
+        return 0;
+    const int st = P->stencil ? 1 : 0, most = (st ? 4 : 2) * P->nsm;
+    switch (P->prob.lattice) {
+    case PKR_D1Q5: P->resident = resident_form<D1Q5>(P->V, st, P->nsm, most); break;
+    case PKR_D1Q9: P->resident = resident_form<D1Q9>(P->V, st, P->nsm, most); break;
+    case PKR_D1Q13: P->resident = resident_form<D1Q13>(P->V, st, P->nsm, most); break;
+    case PKR_D2Q25: P->resident = resident_form<D2Q25>(P->V, st, P->nsm, most); break;
+    case PKR_D2Q81: P->resident = resident_form<D2Q81>(P->V, st, P->nsm, most); break;
+    case PKR_D2Q169: P->resident = resident_form<D2Q169>(P->V, st, P->nsm, most); break;
+    case PKR_D3Q19: P->resident = resident_form<D3Q19>(P->V, st, P->nsm, most); break;
+    case PKR_D3Q111: P->resident = resident_form<D3Q111>(P->V, st, P->nsm, most); break;
+    }
+    return P->resident;
+}
+
+int launch_resident_steps(pkr_plan* P, int form, int nsteps, double tol, int kind)
+{
+    CoopArgs a{};
+    if (P->stencil) {
+        a.P[0] = P->Ps[P->cur];
+        a.P[1] = P->Ps[P->cur ^ 1];
+        a.S = P->St;
+    } else {
+        a.P[0] = static_cast<double*>(P->pop[P->cur]);
+        a.P[1] = static_cast<double*>(P->pop[P->cur ^ 1]);
+        a.P[2] = static_cast<double*>(P->pop3);
+        a.S = static_cast<const double*>(P->S);
+        a.Phi = P->Phi;
+    }
+    a.partials = P->partials;   // 8 doubles per tile: within the sweep's scratch
+    a.counter = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(P->ctl) + 64);
+    a.ctl = P->ctl;
+    a.tol = tol;
+    a.V = P->V;
+    a.nx = (int)P->prob.n[0];
+    a.ny = (int)P->prob.n[1];
+    a.nz = (int)P->prob.n[2];
+    a.small = P->small;
+    a.kind = kind;
+    a.nsteps = nsteps;
+    int rc = -1;
+    switch (P->prob.lattice) {
+    case PKR_D1Q5: rc = launch_resident<D1Q5>(form, a, P->c64, P->stream); break;
+    case PKR_D1Q9: rc = launch_resident<D1Q9>(form, a, P->c64, P->stream); break;
+    case PKR_D1Q13: rc = launch_resident<D1Q13>(form, a, P->c64, P->stream); break;
+    case PKR_D2Q25: rc = launch_resident<D2Q25>(form, a, P->c64, P->stream); break;
+    case PKR_D2Q81: rc = launch_resident<D2Q81>(form, a, P->c64, P->stream); break;
+    case PKR_D2Q169: rc = launch_resident<D2Q169>(form, a, P->c64, P->stream); break;
+    case PKR_D3Q19: rc = launch_resident<D3Q19>(form, a, P->c64, P->stream); break;
+    case PKR_D3Q111: rc = launch_resident<D3Q111>(form, a, P->c64, P->stream); break;
+    }
+    return rc == 0 ? PKR_OK : PKR_ECUDA;
+}
+
+// Memory of a resident run (its rule's state, and the sweep's third array).
+bool resident_ready(pkr_plan* P, int form)
+{
+    if (!P->ctl && alloc_ctl(P) != PKR_OK) return false;
+    if (form == 3 && !P->pop3 &&
+        cudaMalloc(&P->pop3, (size_t)P->lat.Q * (size_t)P->V * 8 + 16) != cudaSuccess) {
+        cudaGetLastError();
+        P->pop3 = nullptr;
+        return false;
+    }
+    return true;
+}
+
+// The host's view after a resident launch that kept `ran` steps.
+void resident_advance(pkr_plan* P, int form, int64_t ran)
+{
+    P->launches += ran;
+    if (form != 3) {
+        if (ran & 1) P->cur ^= 1;
+        P->Phi = P->Ps[P->cur];
+        return;
+    }
+    void* arr[3] = {P->pop[P->cur], P->pop[P->cur ^ 1], P->pop3};
+    const int m = (int)(ran % 3);
+    P->pop[P->cur] = arr[m];
+    P->pop[P->cur ^ 1] = arr[(m + 1) % 3];
+    P->pop3 = arr[(m + 2) % 3];
+    if (P->gexec) {   // captured with the arrays in their old places
+        cudaGraphExecDestroy(P->gexec);
+        P->gexec = nullptr;
+    }
+}
+
 // Capture kGraphSteps check steps, each followed by the stopping rule on the
 // device, as one graph for this plan, array parity, tol and tol kind.  The
 // host view that launch_one advances (parity, step count, Phi) is restored
@@ -425,11 +546,8 @@ constexpr int kGraphSteps = 64;
 int capture_steps(pkr_plan* P, double tol, int tol_kind)
 {
     if (!P->ctl) {
-        if (cudaMalloc((void**)&P->ctl, sizeof(RunCtl)) != cudaSuccess ||
-            cudaMallocHost((void**)&P->hctl, sizeof(RunCtl)) != cudaSuccess) {
-            cudaGetLastError();
-            return PKR_ENOMEM;
-        }
+        const int rc = alloc_ctl(P);
+        if (rc != PKR_OK) return rc;
     }
     if (!P->cap && cudaStreamCreateWithFlags(&P->cap, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
@@ -623,6 +741,7 @@ int plan_create(const pkr_problem* p, void* stream, pkr_plan** out, bool spare)
     for (int k = 0; k < li.dim; ++k)
         if (p->n[k] < li.reach) P->small = 1;
     P->last_residual = -1.0;
+    P->resident = -1;
     // collision coefficients per symmetry class
     P->c64.om1 = 1.0 - omega;
     P->c32.om1 = (float)(1.0 - omega);
@@ -746,6 +865,7 @@ int pkr_plan_destroy(pkr_plan* P)
     if (P->stream || P->pop[0] || P->Ps[0]) cudaStreamSynchronize(P->stream);
     cudaFree(P->pop[0]);
     cudaFree(P->pop[1]);
+    cudaFree(P->pop3);
     cudaFree(P->Ps[0]);
     cudaFree(P->Ps[1]);
     cudaFree(P->St);
@@ -1025,8 +1145,39 @@ int pkr_plan_run(pkr_plan* P, int64_t steps, double tol, int tol_kind, int check
     // applied on the device after each check, and the host reads the outcome
     // once per graph instead of once per step.  Same steps, same stopping step.
     if (K == 1 && tol > 0.0 && P->prob.precision == PKR_FP64 && steps >= kGraphSteps) {
-        bool ok = true;
-        if (!P->gexec || P->gcur != P->cur || P->gtol != tol || P->gkind != tol_kind)
+        // small grids: all steps in a few resident launches
+        const int form = resident_of(P);
+        if (form > 0 && resident_ready(P, form)) {
+            *P->hctl = RunCtl{0, PKR_OK, -1, 0, INFINITY, P->last_residual};
+            while (done < steps && !stopped) {
+                const int64_t n = steps - done < kResidentSteps ? steps - done : kResidentSteps;
+                PKR_CK(cudaMemcpyAsync(P->ctl, P->hctl, sizeof(RunCtl), cudaMemcpyHostToDevice,
+                                       P->stream));
+                PKR_CK(cudaMemsetAsync(reinterpret_cast<char*>(P->ctl) + 64, 0,
+                                       sizeof(unsigned int), P->stream));
+                if (launch_resident_steps(P, form, (int)n, tol, tol_kind) != PKR_OK) {
+                    if (done > 0) return PKR_ECUDA;
+                    cudaGetLastError();   // not launched: step as other plans do
+                    P->resident = 0;
+                    break;
+                }
+                PKR_CK(cudaMemcpyAsync(P->hctl, P->ctl, sizeof(RunCtl), cudaMemcpyDeviceToHost,
+                                       P->stream));
+                PKR_CK(cudaStreamSynchronize(P->stream));
+                const RunCtl c = *P->hctl;
+                if (c.status == PKR_ECUDA) return PKR_ECUDA;
+                resident_advance(P, form, (int64_t)c.done_at + 1);
+                done += (int64_t)c.done_at + 1;
+                P->last_residual = c.last_res;
+                nchecks = c.nchecks;
+                min_res = c.min_res;
+                status = c.status;
+                stopped = c.stop != 0;
+            }
+        }
+        bool ok = !stopped && done < steps;
+        if (!ok) {
+        } else if (!P->gexec || P->gcur != P->cur || P->gtol != tol || P->gkind != tol_kind)
             ok = capture_steps(P, tol, tol_kind) == PKR_OK;
         if (ok) {
             *P->hctl = RunCtl{0, PKR_OK, -1, 0, INFINITY, P->last_residual};

@@ -122,6 +122,18 @@ struct RunCtl {
     double last_res;  // last checked residual
 };
 
+// A resident run (pkr_resident.cuh): up to nsteps check steps in one launch.
+struct CoopArgs {
+    double* P[3];            // stencil: the two Phi arrays; sweep: three population arrays
+    const double* S;         // St (stencil) or S (sweep)
+    double* Phi;             // sweep: density out
+    double* partials;        // 8 doubles per tile
+    unsigned int* counter;   // zero at launch
+    RunCtl* ctl;
+    double tol;
+    int64_t V;
+    int nx, ny, nz, small, kind, nsteps;
+};
 
 // Source preparation and reductions (pkr_kernels.cu).
 int launch_rho_partials(const double* rho, int64_t V, double* partials, int nblocks,

@@ -1427,6 +1427,7 @@ int occupancy_h16(int variant, int* blocks, int* tiles_per_block)
 #include "pkr_stencil.cuh"
 #include "pkr_sweep_pair.cuh"
 #include "pkr_sweep_ws.cuh"
+#include "pkr_resident.cuh"
 
 namespace pkr {
 
@@ -1521,6 +1522,8 @@ int batch_variant_count_t() { return Variants<L>::N; }
     template int launch_stencil<L>(const double*, double*, const double*, const Coefs<double>&,  \
                                    int64_t, int, int, int, int, int, double*, int, int, void*,  \
                                    const int*);                                                 \
+    template int resident_form<L>(int64_t, int, int, int);                                   \
+    template int launch_resident<L>(int, const CoopArgs&, const Coefs<double>&, void*);      \
     template int launch_batch_t<L, double>(int, BatchState*, int, int, void*);               \
     template int launch_batch_t<L, float>(int, BatchState*, int, int, void*);                \
     template int launch_batch_t<L, long long>(int, BatchState*, int, int, void*);            \
