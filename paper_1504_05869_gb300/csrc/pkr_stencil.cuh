@@ -83,6 +83,17 @@ struct Neighbours {
                 zo[d + RC] = (small ? wrap_any(z - d, nz) : wrap_near(z - d, nz)) * nxy;
         }
     }
+    // Keeps the compiler from forming all Q sums of at() ahead of a loop that
+    // uses them (it would spill them).
+    __device__ __forceinline__ void hold()
+    {
+#pragma unroll
+        for (int d = 0; d < W; ++d) asm volatile("" : "+r"(xs[d]));
+        if constexpr (WY > 1) {
+#pragma unroll
+            for (int d = 0; d < W; ++d) asm volatile("" : "+r"(yo[d]));
+        }
+    }
     // flat index of x - v_i
     template <int i>
     __device__ __forceinline__ int at() const
