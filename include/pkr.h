@@ -80,9 +80,10 @@ typedef enum pkr_lattice {
  * (set before each step so that the step's largest value has 4x headroom),
  * arithmetic in binary32, source in binary32; accurate to ~1e-4 of Phi.
  * Where nx is a multiple of 64 and no edge is below the lattice's reach, the
- * sweep gives each lane two adjacent sites (variant 1, the default there;
- * variant 0 keeps one site per lane); both give the same Phi bit for bit
- * between residual checks.
+ * sweep gives each lane two adjacent sites, or four where nx is a multiple of
+ * 128 and the grid has a 128-site tile for every resident warp (variant 1, the
+ * default there; variant 0 keeps one site per lane); all give the same Phi bit
+ * for bit between residual checks.
  * MIXED16 (pkr_solve only): binary16 to PKR_MIXED16_SWITCH_TOL, binary32 to
  * PKR_MIXED_SWITCH_TOL, then binary64 to tol.
  * A reduced-precision rung also hands over at its rounding floor, which can
@@ -157,7 +158,7 @@ typedef struct pkr_stats {
     int32_t variant;         /* sweep geometry that ran (its last plan, for a precision
                                 ladder): an index into the list pkr_variant_count counts
                                 (pkr_batch_variant_count for a context's request; binary16:
-                                0 one site per lane, 1 two); -1 when no population sweep
+                                0 one site per lane, 1 several); -1 when no population sweep
                                 ran (scalar stencil, pkr_fixed_point_fft) */
 } pkr_stats;
 

@@ -188,7 +188,7 @@ struct pkr_plan {
     // (pkr_plan_run returns PKR_OK) once the residual, below this cap, stops
     // falling from one check to the next (the storage's rounding floor)
     double stall_cap;
-    bool h16pairs;      // binary16 storage: the two-sites-per-lane sweep applies
+    bool h16pairs;      // binary16 storage: the several-sites-per-lane sweeps apply
     bool xpairs;        // other storage: the aligned x-pairs sweep applies
     cudaStream_t stream;
     int device, grid, red_blocks, elem, small, variant, nsm;
@@ -270,6 +270,15 @@ int launch_stencil_step(pkr_plan* P, const double* in, double* out, const double
     return rc == 0 ? PKR_OK : PKR_ECUDA;
 }
 
+// binary16: form of the sweep that variant `variant` of this plan runs.
+// Variant 1 takes four sites per lane on x rows of whole 128-site tiles once
+// they give every resident warp (six per SM) a tile, else two.
+int h16_form(const pkr_plan* P, int variant)
+{
+    if (variant != 1 || !P->h16pairs) return 0;
+    return P->prob.n[0] % 128 == 0 && P->V / 128 >= (int64_t)6 * P->nsm ? 2 : 1;
+}
+
 int launch_one(pkr_plan* P, int mode, bool zero_in)
 {
     if (P->stencil) {
@@ -315,7 +324,7 @@ int launch_one(pkr_plan* P, int mode, bool zero_in)
     a.oflow = P->h16of;
     a.stop = P->stop_arg;
     if (pr == PKR_FP16) {
-        const int vh = (vr == 1 && P->h16pairs) ? 1 : 0;
+        const int vh = h16_form(P, vr);
         switch (P->prob.lattice) {
         case PKR_D1Q5: rc = launch_sweep_h16<D1Q5>(vh, a, c, P->grid, P->stream); break;
         case PKR_D1Q9: rc = launch_sweep_h16<D1Q9>(vh, a, c, P->grid, P->stream); break;
@@ -401,7 +410,8 @@ int set_variant(pkr_plan* P, int variant)
         !P->xpairs)
         variant = 2;
     int bps = 0, tpb = 1;
-    if (occupancy(variant, P->prob.lattice, P->prob.precision, &bps, &tpb) != 0 || bps < 1)
+    const int form = P->prob.precision == PKR_FP16 ? h16_form(P, variant) : variant;
+    if (occupancy(form, P->prob.lattice, P->prob.precision, &bps, &tpb) != 0 || bps < 1)
         return PKR_ECUDA;
     const int64_t nbt = (P->ntiles + tpb - 1) / tpb;
     int64_t grid = (int64_t)P->nsm * bps;

@@ -1180,16 +1180,52 @@ __device__ __forceinline__ unsigned int prmt(unsigned int a, unsigned int b, uns
     return r;
 }
 
-// Lane's pair of a velocity from its slot (sw: this lane's word, 4 l), after
-// the repack: one aligned word, low half the even site, high half the odd one.
-__device__ __forceinline__ float2 h16_word(uint32_t sw)
+// Two binary32 values in one 64-bit register pair, added and multiplied by one
+// instruction each; every half rounds as the scalar operation does.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi)
 {
-    const unsigned int w = lds_b32(sw);
-    return __half22float2(*reinterpret_cast<const __half2*>(&w));
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// max(m, |x|, |y|)
+__device__ __forceinline__ float max3_abs(float m, float x, float y)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(fabsf(x)), "f"(fabsf(y)));
+    return r;
 }
 
-template <class L, int TILES>
-__global__ void __launch_bounds__(TILES * 32, 7)   // 128 registers: 7 blocks per SM
+// Lane's pair of a velocity from its slot (sw: this lane's word, 4 l), after
+// the repack: one aligned word, low half the even site, high half the odd one.
+__device__ __forceinline__ f32x2 h16_pair(uint32_t sw)
+{
+    const unsigned int w = lds_b32(sw);
+    const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&w));
+    return pack2(v.x, v.y);
+}
+
+template <class L, int TILES, int MINB>
+__global__ void __launch_bounds__(TILES * 32, MINB)
 sweep_h16p_kernel(const SweepArgs a, const Coefs<float> c)
 {
     constexpr int Q = L::Q;
@@ -1222,46 +1258,51 @@ sweep_h16p_kernel(const SweepArgs a, const Coefs<float> c)
     double rd2 = 0.0, rn2 = 0.0, rmx = 0.0, rms = 0.0;
     float pmax = 0.f;
     const int nt = gridDim.x * TILES;
-    for (int tile = blockIdx.x * TILES + sub; tile < ntiles; tile += nt) {
+    const int nb = a.zero_in ? 0 : 4;
+    // the tile whose slots are being filled: row offsets, the first x, and the
+    // lane's word of the run for each x displacement -R..R (the first word of
+    // a run is (x0 - vx) rounded down to even, halved)
+    int yo[W], zo[W], wl[W], x0 = 0;
+    auto locate = [&](int tile) {
         const int s0 = tile * 64;              // first site: x0 = s0 mod nx, even
         const int r = (int)((unsigned)s0 / (unsigned)nx);
-        const int x0 = s0 - r * nx;
+        x0 = s0 - r * nx;
         const int z = (int)((unsigned)r / (unsigned)ny);
         const int y = r - z * ny;
-        int yo[W], zo[W];
         static_for<0, W>([&](auto DI) {
             constexpr int d = decltype(DI)::value - RC;
             yo[d + RC] = wrap_off<d>(y, ny) * nw;
             zo[d + RC] = wrap_off<d>(z, nz) * (ny * nw);
+            int w = ((x0 - d) >> 1) + lane;    // arithmetic shift: floor
+            wl[d + RC] = w < 0 ? w + nw : (w >= nw ? w - nw : w);
         });
-        const int nb = a.zero_in ? 0 : 4;
-        // lane's word of the run for each x displacement -R..R (the first
-        // word of a run is (x0 - vx) rounded down to even, halved)
-        int wl[W];
-        static_for<0, W>([&](auto DI) {
-            constexpr int vx = decltype(DI)::value - RC;
-            int w = ((x0 - vx) >> 1) + lane;   // arithmetic shift: floor
-            wl[vx + RC] = w < 0 ? w + nw : (w >= nw ? w - nw : w);
-        });
-        const unsigned int* plane = A;          // plane i, advanced per velocity
-        static_for<0, Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            constexpr int vx = vx_of<L>(i);
-            constexpr int oy = vy_of<L>(i) + RC;
-            constexpr int oz = vz_of<L>(i) + RC;
-            const unsigned int* row = plane + (zo[oz] + yo[oy]);
-            plane += Vw;
-            cp_async<4>(sw + (uint32_t)(i * SW), row + wl[vx + RC], nb);
-            if constexpr (vx & 1) {
-                // word 32 of an odd run, copied by lane 0; the other lanes
-                // issue the same instruction with nothing to read, into a
-                // word of their own (no branch in the unrolled pull)
-                int w1 = ((x0 - vx) >> 1) + 32;
-                w1 = w1 >= nw ? w1 - nw : w1;
-                cp_async<4>(lane == 0 ? slot + (uint32_t)(i * SW + 128) : dummy, row + w1,
-                            lane == 0 ? nb : 0);
-            }
-        });
+    };
+    auto pull = [&](auto I) {
+        constexpr int i = decltype(I)::value;
+        constexpr int vx = vx_of<L>(i);
+        const unsigned int* row =
+            A + ((int64_t)i * Vw + (zo[vz_of<L>(i) + RC] + yo[vy_of<L>(i) + RC]));
+        cp_async<4>(sw + (uint32_t)(i * SW), row + wl[vx + RC], nb);
+        if constexpr (vx & 1) {
+            // word 32 of an odd run, copied by lane 0; the other lanes
+            // issue the same instruction with nothing to read, into a
+            // word of their own (no branch in the unrolled pull)
+            int w1 = ((x0 - vx) >> 1) + 32;
+            w1 = w1 >= nw ? w1 - nw : w1;
+            cp_async<4>(lane == 0 ? slot + (uint32_t)(i * SW + 128) : dummy, row + w1,
+                        lane == 0 ? nb : 0);
+        }
+    };
+    const int first = blockIdx.x * TILES + sub;
+    if (first < ntiles) {
+        locate(first);
+        static_for<0, Q>(pull);
+    }
+    for (int tile = first; tile < ntiles; tile += nt) {
+        const int s = tile * 64 + 2 * lane;
+        const float2 S2 = *reinterpret_cast<const float2*>(S + s);
+        const bool more = tile + nt < ntiles;
+        if (more) locate(tile + nt);
         cp_async_wait_all();
         __syncwarp();
         // repack every odd run in place into aligned pairs: word l := high
@@ -1280,50 +1321,46 @@ sweep_h16p_kernel(const SweepArgs a, const Coefs<float> c)
 
         // density: per site the four interleaved binary32 partials of
         // density_fixed_f32 (velocity k to partial k mod 4, the last Q mod 4
-        // to partial 0), then the array's scale
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, b0 = 0.f, b1 = 0.f, b2 = 0.f, b3 = 0.f;
+        // to partial 0), then the array's scale; both sites in one packed add
+        f32x2 p0 = 0, p1 = 0, p2 = 0, p3 = 0;
 #pragma unroll 2
         for (int k = 0; k + 3 < Q; k += 4) {
-            const float2 v0 = h16_word(sw + (uint32_t)((k + 0) * SW));
-            const float2 v1 = h16_word(sw + (uint32_t)((k + 1) * SW));
-            const float2 v2 = h16_word(sw + (uint32_t)((k + 2) * SW));
-            const float2 v3 = h16_word(sw + (uint32_t)((k + 3) * SW));
-            a0 += v0.x; b0 += v0.y;
-            a1 += v1.x; b1 += v1.y;
-            a2 += v2.x; b2 += v2.y;
-            a3 += v3.x; b3 += v3.y;
+            p0 = add2(p0, h16_pair(sw + (uint32_t)((k + 0) * SW)));
+            p1 = add2(p1, h16_pair(sw + (uint32_t)((k + 1) * SW)));
+            p2 = add2(p2, h16_pair(sw + (uint32_t)((k + 2) * SW)));
+            p3 = add2(p3, h16_pair(sw + (uint32_t)((k + 3) * SW)));
         }
 #pragma unroll
-        for (int k = Q - Q % 4; k < Q; ++k) {
-            const float2 v = h16_word(sw + (uint32_t)(k * SW));
-            a0 += v.x; b0 += v.y;
-        }
-        const float PhiA = ((a0 + a1) + (a2 + a3)) * sr;
-        const float PhiB = ((b0 + b1) + (b2 + b3)) * sr;
+        for (int k = Q - Q % 4; k < Q; ++k) p0 = add2(p0, h16_pair(sw + (uint32_t)(k * SW)));
+        const float2 sum = unpack2(add2(add2(p0, p1), add2(p2, p3)));
+        const float PhiA = sum.x * sr;
+        const float PhiB = sum.y * sr;
         // the written array's scale inv_sw is a power of two, so it enters the
         // relaxation factor and the per-class terms exactly: the products
         // below are the stored values p / sc, bit for bit those of p * inv_sw
         const float om1w = c.om1 * sr * inv_sw;
-        const int s = s0 + 2 * lane;
-        const float2 S2 = *reinterpret_cast<const float2*>(S + s);
+        const f32x2 om2 = pack2(om1w, om1w);
         const float SxA = (float)((double)S2.x + a.soff);
         const float SxB = (float)((double)S2.y + a.soff);
         unsigned int* dst = B + (s >> 1);       // plane i's word of the pair, per velocity
         static_for<0, NC>([&](auto CI) {
             constexpr int cl = decltype(CI)::value;
             constexpr int i0 = cls_begin<L>(cl), i1 = cls_begin<L>(cl + 1);
-            const float eA = fmaf(c.wphi[cl], PhiA, c.chi[cl] * SxA) * inv_sw;
-            const float eB = fmaf(c.wphi[cl], PhiB, c.chi[cl] * SxB) * inv_sw;
+            const f32x2 e = pack2(fmaf(c.wphi[cl], PhiA, c.chi[cl] * SxA) * inv_sw,
+                                  fmaf(c.wphi[cl], PhiB, c.chi[cl] * SxB) * inv_sw);
 #pragma unroll 4
             for (int i = i0; i < i1; ++i) {
-                const float2 v = h16_word(sw + (uint32_t)(i * SW));
-                const float qA = fmaf(om1w, v.x, eA);   // p / sc of the written array
-                const float qB = fmaf(om1w, v.y, eB);
-                pmax = fmaxf(pmax, fmaxf(fabsf(qA), fabsf(qB)));
-                const __half2 h = __floats2half2_rn(qA, qB);
+                // p / sc of the written array
+                const float2 q = unpack2(fma2(om2, h16_pair(sw + (uint32_t)(i * SW)), e));
+                pmax = max3_abs(pmax, q.x, q.y);
+                const __half2 h = __floats2half2_rn(q.x, q.y);
                 __stcs(dst, *reinterpret_cast<const unsigned int*>(&h));
                 dst += Vw;
             }
+            // the class's slots take the next tile: its copies are in flight
+            // while the other classes and the next tile's repack run
+            __syncwarp();
+            if (more) static_for<i0, i1>(pull);
         });
         if (a.mode != kPlain) {
             const double phA = (double)PhiA, phB = (double)PhiB;
@@ -1340,7 +1377,6 @@ sweep_h16p_kernel(const SweepArgs a, const Coefs<float> c)
             }
             *reinterpret_cast<double2*>(a.Phi + s) = make_double2(phA, phB);
         }
-        __syncwarp();
     }
 
     // pmax holds max |p| / sc (the stored magnitudes): back to max |p|, exactly
@@ -1387,38 +1423,51 @@ sweep_h16p_kernel(const SweepArgs a, const Coefs<float> c)
     }
 }
 
-// binary16 geometries: 0 one site per lane (any grid), 1 two sites per lane
-// (nx a multiple of 64 and no edge below the reach; the plan checks).
+}  // namespace pkr
+
+#include "pkr_sweep_h16w.cuh"
+
+namespace pkr {
+
+// binary16 forms: 0 one site per lane (any grid), 1 two sites per lane (nx a
+// multiple of 64 and no edge below the reach; the plan checks), 2 four sites
+// per lane (nx a multiple of 128).  Tiles per block, measured at 256 x 256 x
+// 192, D3Q111: form 1, 2 tiles and 6 blocks per SM 9.90 GLUPS, 7 blocks (128
+// registers) 9.25; form 2, 2 tiles 11.51, 1 tile 10.41, 3 tiles 11.30, 7 tiles
+// 9.93.
 constexpr int kH16Tiles = 2;
 template <class L>
-constexpr size_t h16_smem(int variant)
+constexpr size_t h16_smem(int form)
 {
-    return variant == 1 ? (size_t)kH16Tiles * (L::Q * 33 * 4 + 32 * 4)
-                        : (size_t)kH16Tiles * L::Q * 32 * 4;
+    return form == 2 ? H16w<L>::smem_bytes(kH16Tiles)
+           : form == 1 ? (size_t)kH16Tiles * (L::Q * 33 * 4 + 32 * 4)
+                       : (size_t)kH16Tiles * L::Q * 32 * 4;
+}
+template <class L>
+auto h16_kernel(int form)
+{
+    return form == 2 ? sweep_h16w_kernel<L, kH16Tiles>
+           : form == 1 ? sweep_h16p_kernel<L, kH16Tiles, 6>
+                       : sweep_h16_kernel<L, kH16Tiles>;
 }
 
 template <class L>
-int launch_sweep_h16(int variant, const SweepArgs& a, const void* coefs, int grid, void* stream)
+int launch_sweep_h16(int form, const SweepArgs& a, const void* coefs, int grid, void* stream)
 {
     const Coefs<float>& c = *static_cast<const Coefs<float>*>(coefs);
-    if (variant == 1)
-        sweep_h16p_kernel<L, kH16Tiles><<<grid, kH16Tiles * 32, h16_smem<L>(1),
-                                         (cudaStream_t)stream>>>(a, c);
-    else
-        sweep_h16_kernel<L, kH16Tiles><<<grid, kH16Tiles * 32, h16_smem<L>(0),
-                                        (cudaStream_t)stream>>>(a, c);
+    h16_kernel<L>(form)<<<grid, kH16Tiles * 32, h16_smem<L>(form), (cudaStream_t)stream>>>(a, c);
     return (int)cudaGetLastError();
 }
 
 template <class L>
-int occupancy_h16(int variant, int* blocks, int* tiles_per_block)
+int occupancy_h16(int form, int* blocks, int* tiles_per_block)
 {
-    const size_t smem = h16_smem<L>(variant);
-    auto kern = variant == 1 ? sweep_h16p_kernel<L, kH16Tiles> : sweep_h16_kernel<L, kH16Tiles>;
+    const size_t smem = h16_smem<L>(form);
+    auto kern = h16_kernel<L>(form);
     cudaError_t e = set_sweep_smem(kern, smem);
     if (e != cudaSuccess) return (int)e;
-    // tiles_per_block counts 32-site tiles: a two-site tile is two of them
-    *tiles_per_block = variant == 1 ? 2 * kH16Tiles : kH16Tiles;
+    // tiles_per_block counts 32-site tiles
+    *tiles_per_block = (form == 2 ? 4 : form == 1 ? 2 : 1) * kH16Tiles;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kern, kH16Tiles * 32, smem);
 }
 

@@ -1,0 +1,60 @@
+"""Sweeps with several sites per lane against the one-site forms.
+
+binary16 with four sites per lane (x rows of whole 128-site tiles) and binary32
+with two (x rows of whole 64-site pairs) do per site what the one-site kernels
+do, in the same order: the same Phi bit for bit between residual checks.  A
+check's sums run in another order, and binary32 and binary16 steps take the
+mass it measures out through the source, so after checks the two agree to
+rounding of the storage."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pk():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1504_05869_gb300 as pk
+    return pk
+
+
+def _run(pk, rho, lattice, order, precision, variant, steps, every):
+    import torch
+    prob = pk.problem(lattice, rho.shape, order, tau_lb=1.7, max_sweeps=1000, precision=precision,
+                      variant=variant)
+    phi = torch.empty_like(rho)
+    with pk.Plan(prob) as P:
+        P.load_source(rho)
+        _, st = P.run(steps, check_every=every)
+        P.phi(phi)
+    return phi, st
+
+
+def _rho(shape, seed):
+    import torch
+    g = torch.Generator().manual_seed(seed)
+    return torch.randn(shape, generator=g, dtype=torch.float64).cuda()
+
+
+# one tile per row (both halos wrap), several, reaches 1 to 6, tile counts that
+# leave the last block part full; all with a tile for every resident warp
+@pytest.mark.parametrize("lattice,order,shape", [
+    ("D3Q111", 5, (31, 30, 128)), ("D3Q111", 5, (7, 67, 256)), ("D3Q111", 5, (3, 103, 384)),
+    ("D3Q19", 1, (33, 29, 128)), ("D2Q25", 3, (913, 128)), ("D2Q81", 5, (457, 256)),
+    ("D2Q169", 7, (915, 128)), ("D1Q13", 7, (128 * 913,)),
+])
+def test_binary16_four_sites_per_lane(pk, lattice, order, shape):
+    import torch
+    rho = _rho(shape, 3)
+    for steps, every in ((7, 1000), (8, 4)):
+        one, _ = _run(pk, rho, lattice, order, "fp16", 0, steps, every)
+        four, st = _run(pk, rho, lattice, order, "fp16", -1, steps, every)
+        assert st["variant"] == 1
+        if every > steps:
+            assert torch.equal(one, four)
+        else:
+            assert float((one - four).norm() / one.norm()) <= 1e-6
