@@ -158,6 +158,8 @@ def kernel_label(pk, variant):
         return f"sweep_staged_kernel<{LATTICE},{T}>"
     if nv - variant <= 2 and nv - nb == 3:
         form = "early refill" if variant == nv - 1 else "refill after the pair"
+        if PRECISION == "fp32" and variant == nv - 1:
+            return f"sweep_wide_kernel<{LATTICE}>"
         return f"sweep_pair_kernel<{LATTICE},{T},G=2> ({form})"
     return f"sweep_ws_kernel<{LATTICE},{T}>"
 

@@ -191,7 +191,7 @@ int pkr_tau_from_knudsen(int lattice, double knudsen, const int64_t n[3], double
  * warps filling a ring of tile slots, groups of compute warps draining it)
  * and the two aligned x-pairs ones (64-site x pairs copied from aligned runs;
  * the second refills each symmetry class's rows for the block's next pair as
- * soon as that class is relaxed).  The x-pairs variants apply to grids whose
+ * soon as that class is relaxed; in binary32 it gives each lane two sites).  The x-pairs variants apply to grids whose
  * x edge is a multiple of 64 and whose every edge is at least the reach;
  * asked for on other grids, a plan takes the staged 2 x 2 geometry instead.
  * Host only; < 0 for an unknown lattice. */

@@ -1474,6 +1474,7 @@ int occupancy_h16(int form, int* blocks, int* tiles_per_block)
 }  // namespace pkr
 
 #include "pkr_stencil.cuh"
+#include "pkr_sweep_wide.cuh"
 #include "pkr_sweep_pair.cuh"
 #include "pkr_sweep_ws.cuh"
 #include "pkr_resident.cuh"

@@ -281,14 +281,21 @@ sweep_pair_kernel(const SweepArgs a, const Coefs<typename AccType<T>::type> c)
     }
 }
 
+// (binary32 runs its early-refill form with two sites per lane:
+// pkr_sweep_wide.cuh, 6.4 against 5.6 GLUPS)
 template <class L, typename T, int K>
 int launch_pair_variant(const SweepArgs& a, const void* coefs, int grid, void* stream)
 {
     using R = typename AccType<T>::type;
     constexpr int G = PairVariant<L>::groups(K);
     constexpr bool EARLY = PairVariant<L>::early_refill(K);
-    sweep_pair_kernel<L, T, G, EARLY><<<grid, 64 * G, Pair<L, T>::smem_bytes(), (cudaStream_t)stream>>>(
-        a, *static_cast<const Coefs<R>*>(coefs));
+    const Coefs<R>& c = *static_cast<const Coefs<R>*>(coefs);
+    if constexpr (EARLY && std::is_same<T, float>::value)
+        sweep_wide_kernel<L><<<grid, Wide<L>::THREADS, Wide<L>::smem_bytes(),
+                               (cudaStream_t)stream>>>(a, c);
+    else
+        sweep_pair_kernel<L, T, G, EARLY><<<grid, 64 * G, Pair<L, T>::smem_bytes(),
+                                            (cudaStream_t)stream>>>(a, c);
     return (int)cudaGetLastError();
 }
 
@@ -297,12 +304,20 @@ int occupancy_pair_variant(int* blocks, int* tiles_per_block)
 {
     constexpr int G = PairVariant<L>::groups(K);
     constexpr bool EARLY = PairVariant<L>::early_refill(K);
-    auto kern = sweep_pair_kernel<L, T, G, EARLY>;
-    const size_t smem = Pair<L, T>::smem_bytes();
-    cudaError_t e = set_sweep_smem(kern, smem);
-    if (e != cudaSuccess) return (int)e;
-    *tiles_per_block = 2;
-    return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kern, 64 * G, smem);
+    if constexpr (EARLY && std::is_same<T, float>::value) {
+        cudaError_t e = set_sweep_smem(sweep_wide_kernel<L>, Wide<L>::smem_bytes());
+        if (e != cudaSuccess) return (int)e;
+        *tiles_per_block = 2 * Wide<L>::PAIRS;
+        return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            blocks, sweep_wide_kernel<L>, Wide<L>::THREADS, Wide<L>::smem_bytes());
+    } else {
+        auto kern = sweep_pair_kernel<L, T, G, EARLY>;
+        const size_t smem = Pair<L, T>::smem_bytes();
+        cudaError_t e = set_sweep_smem(kern, smem);
+        if (e != cudaSuccess) return (int)e;
+        *tiles_per_block = 2;
+        return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kern, 64 * G, smem);
+    }
 }
 
 }  // namespace pkr

@@ -58,3 +58,22 @@ def test_binary16_four_sites_per_lane(pk, lattice, order, shape):
             assert torch.equal(one, four)
         else:
             assert float((one - four).norm() / one.norm()) <= 1e-6
+
+
+@pytest.mark.parametrize("lattice,order,shape", [
+    ("D3Q111", 5, (5, 7, 64)), ("D3Q111", 5, (37, 33, 64)), ("D3Q111", 5, (9, 11, 192)),
+    ("D3Q111", 5, (3, 3, 128)), ("D2Q81", 5, (41, 128)), ("D2Q169", 7, (7, 64)),
+    ("D2Q169", 7, (13, 320)),
+])
+def test_binary32_two_sites_per_lane(pk, lattice, order, shape):
+    import torch
+    last = pk._pkr.pkr_variant_count(pk.LATTICES[lattice]) - 1
+    rho = _rho(shape, 4)
+    for steps, every in ((7, 1000), (8, 4)):
+        pair, _ = _run(pk, rho, lattice, order, "fp32", last - 1, steps, every)
+        wide, st = _run(pk, rho, lattice, order, "fp32", last, steps, every)
+        assert st["variant"] == last
+        if every > steps:
+            assert torch.equal(pair, wide)
+        else:
+            assert float((pair - wide).norm() / pair.norm()) <= 1e-6
