@@ -2,8 +2,8 @@
 //
 // A context owns the device-resident batch state: one descriptor per live
 // grid, the batch-wide tile partials and per-grid residuals.  One K-step
-// "window" is a captured CUDA graph: K x (persistent batch sweep, step
-// counter increment), the per-grid residual reduction and the copy of the
+// "window" is a captured CUDA graph: K persistent batch sweeps, the per-grid
+// residual reduction (which moves the step counter on by K) and the copy of the
 // residuals to pinned host memory.  Between windows the host admits queued
 // requests that fit the HBM budget (first fit; source preparation on the
 // context's stream; they start at the window boundary) and retires the grids
@@ -33,7 +33,7 @@
 #include "pkr_internal.h"
 
 namespace pkr {
-template <class L, typename T> int launch_batch_t(int, BatchState*, int, int, void*);
+template <class L, typename T> int launch_batch_t(int, BatchState*, int, int, int, void*);
 template <class L, typename T> int batch_occupancy_t(int, int*);
 template <class L> int batch_variant_count_t();
 
@@ -57,11 +57,11 @@ int batch_variant_count(int lattice)
 }
 
 template <class L>
-int batch_launch_l(int prec, int var, BatchState* st, int K, int grid, void* s)
+int batch_launch_l(int prec, int var, BatchState* st, int k, int phase, int grid, void* s)
 {
-    if (prec == PKR_FP64) return launch_batch_t<L, double>(var, st, K, grid, s);
-    if (prec == PKR_FX64) return launch_batch_t<L, long long>(var, st, K, grid, s);
-    return launch_batch_t<L, float>(var, st, K, grid, s);
+    if (prec == PKR_FP64) return launch_batch_t<L, double>(var, st, k, phase, grid, s);
+    if (prec == PKR_FX64) return launch_batch_t<L, long long>(var, st, k, phase, grid, s);
+    return launch_batch_t<L, float>(var, st, k, phase, grid, s);
 }
 template <class L>
 int batch_occ_l(int prec, int var, int* b)
@@ -73,18 +73,18 @@ int batch_occ_l(int prec, int var, int* b)
 
 }  // namespace
 
-int launch_batch_step(int lattice, int precision, int variant, BatchState* st, int K, int grid,
-                      void* stream)
+int launch_batch_step(int lattice, int precision, int variant, BatchState* st, int k, int phase,
+                      int grid, void* stream)
 {
     switch (lattice) {
-    case PKR_D1Q5: return batch_launch_l<D1Q5>(precision, variant, st, K, grid, stream);
-    case PKR_D1Q9: return batch_launch_l<D1Q9>(precision, variant, st, K, grid, stream);
-    case PKR_D1Q13: return batch_launch_l<D1Q13>(precision, variant, st, K, grid, stream);
-    case PKR_D2Q25: return batch_launch_l<D2Q25>(precision, variant, st, K, grid, stream);
-    case PKR_D2Q81: return batch_launch_l<D2Q81>(precision, variant, st, K, grid, stream);
-    case PKR_D2Q169: return batch_launch_l<D2Q169>(precision, variant, st, K, grid, stream);
-    case PKR_D3Q19: return batch_launch_l<D3Q19>(precision, variant, st, K, grid, stream);
-    case PKR_D3Q111: return batch_launch_l<D3Q111>(precision, variant, st, K, grid, stream);
+    case PKR_D1Q5: return batch_launch_l<D1Q5>(precision, variant, st, k, phase, grid, stream);
+    case PKR_D1Q9: return batch_launch_l<D1Q9>(precision, variant, st, k, phase, grid, stream);
+    case PKR_D1Q13: return batch_launch_l<D1Q13>(precision, variant, st, k, phase, grid, stream);
+    case PKR_D2Q25: return batch_launch_l<D2Q25>(precision, variant, st, k, phase, grid, stream);
+    case PKR_D2Q81: return batch_launch_l<D2Q81>(precision, variant, st, k, phase, grid, stream);
+    case PKR_D2Q169: return batch_launch_l<D2Q169>(precision, variant, st, k, phase, grid, stream);
+    case PKR_D3Q19: return batch_launch_l<D3Q19>(precision, variant, st, k, phase, grid, stream);
+    case PKR_D3Q111: return batch_launch_l<D3Q111>(precision, variant, st, k, phase, grid, stream);
     }
     return (int)cudaErrorInvalidValue;
 }
@@ -525,15 +525,17 @@ int rebuild(pkr_ctx* C, Lane& L)
 // Queue one window of a lane (K steps + reduction + residual copy).
 int enqueue_window(pkr_ctx* C, Lane& L)
 {
-    for (int k = 0; k < C->K; ++k) {
-        if (launch_batch_step(C->cfg.lattice, L.prec, L.variant, L.d_state, C->K, L.grid,
+    const int K = C->K;
+    for (int k = 0; k < K; ++k) {
+        const int phase = (k == 0 ? kPhaseFirst : 0) | ((k + 2) % K == 0 ? kPhaseWrite : 0) |
+                          (k + 1 == K ? kPhaseCheck : 0);
+        if (launch_batch_step(C->cfg.lattice, L.prec, L.variant, L.d_state, k, phase, L.grid,
                               C->stream) != 0 ||
             (L.prec == PKR_FX64 &&
-             launch_batch_fx_rescale(L.d_state, C->max_grids, C->stream) != 0) ||
-            launch_batch_increment(L.d_state, C->stream) != 0)
+             launch_batch_fx_rescale(L.d_state, k, C->max_grids, C->stream) != 0))
             return PKR_ECUDA;
     }
-    if (launch_batch_reduce(L.d_state, C->max_grids, L.grid_stride, C->stream) != 0 ||
+    if (launch_batch_reduce(L.d_state, K, C->max_grids, L.grid_stride, C->stream) != 0 ||
         cudaMemcpyAsync(L.h_res, L.d_res, (size_t)C->max_grids * 4 * sizeof(double),
                         cudaMemcpyDeviceToHost, C->stream) != cudaSuccess)
         return PKR_ECUDA;
@@ -1070,11 +1072,10 @@ int tune_variant(pkr_ctx* C, Lane& L, int edge)
             int bps = 0;
             if (batch_occupancy(C->cfg.lattice, L.prec, v, &bps) != 0 || bps < 1) continue;
             const int grid = C->nsm * bps;
-            launch_batch_step(C->cfg.lattice, L.prec, v, L.d_state, 1 << 30, grid, C->stream);
+            launch_batch_step(C->cfg.lattice, L.prec, v, L.d_state, 0, 0, grid, C->stream);
             cudaEventRecord(e0, C->stream);
             for (int k = 0; k < 3; ++k)
-                launch_batch_step(C->cfg.lattice, L.prec, v, L.d_state, 1 << 30, grid,
-                                  C->stream);
+                launch_batch_step(C->cfg.lattice, L.prec, v, L.d_state, 0, 0, grid, C->stream);
             cudaEventRecord(e1, C->stream);
             if (cudaEventSynchronize(e1) != cudaSuccess) break;
             float ms = 0.f;

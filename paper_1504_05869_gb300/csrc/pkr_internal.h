@@ -73,7 +73,7 @@ struct BatchState {
     const void* grids;     // BatchGrid<R>[ngrids], sorted by tile_begin
     double* tile_partials; // 4 doubles per batch-wide tile (check steps)
     double* grid_res;      // 4 doubles per grid (after the per-grid reduction)
-    long long step;        // batch step counter (launch index)
+    long long step;        // batch step counter: first step of the window
     int ngrids;
     int ntiles;
 };
@@ -154,14 +154,22 @@ int launch_finalize_check(const double* partials, int nblocks, double* out4, Run
                           double tol, int tol_kind, int j, void* stream);
 
 // Batch engine kernels (sweep_*.cu / pkr_kernels.cu).
-int launch_batch_step(int lattice, int precision, int variant, BatchState* state, int check_every,
+// Step k of a window (0 .. K - 1; state->step is the window's first step);
+// phase: what the position means to every grid of the batch.
+enum BatchPhase {
+    kPhaseFirst = 1,   // first step of a window: the one after a check
+    kPhaseWrite = 2,   // the step before a check writes Phi
+    kPhaseCheck = 4    // last step of a window: residual check
+};
+int launch_batch_step(int lattice, int precision, int variant, BatchState* state, int k, int phase,
                       int grid, void* stream);
 int batch_occupancy(int lattice, int precision, int variant, int* blocks_per_sm);
-int launch_batch_reduce(BatchState* state, int max_grids, int grid_stride_bytes, void* stream);
-int launch_batch_increment(BatchState* state, void* stream);
+// Per-grid residuals after a window of K steps; moves state->step on by K.
+int launch_batch_reduce(BatchState* state, int K, int max_grids, int grid_stride_bytes,
+                        void* stream);
 // 64-bit fixed-point batches: after a step, each grid's rescale (as
 // launch_fx_rescale does for a plan), for the array its next step writes.
-int launch_batch_fx_rescale(BatchState* state, int max_grids, void* stream);
+int launch_batch_fx_rescale(BatchState* state, int k, int max_grids, void* stream);
 int launch_convert(const void* in, int in_precision, void* out, int out_precision, int64_t n,
                    void* stream);
 // out[i*V + x] = in[i*V + x] - shift[i] (storage conversion with a per-plane

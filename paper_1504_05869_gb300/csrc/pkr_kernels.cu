@@ -182,9 +182,10 @@ finalize_check_kernel(const double* __restrict__ partials, int n, double* out4, 
 // Per-grid residual of a batch check step: sums the grid's tile partials in
 // tile order (deterministic), one block per grid.
 __global__ void __launch_bounds__(kRedThreads)
-batch_reduce_kernel(const BatchState* st, int stride_bytes)
+batch_reduce_kernel(BatchState* st, int K, int stride_bytes)
 {
     const int g = blockIdx.x;
+    if (g == 0 && threadIdx.x == 0) st->step += K;   // read by the next window only
     if (g >= st->ngrids) return;
     const unsigned char* base = static_cast<const unsigned char*>(st->grids);
     const size_t off = offsetof(BatchGrid<double>, tile_begin);
@@ -237,8 +238,6 @@ batch_reduce_kernel(const BatchState* st, int stride_bytes)
         if (gd.soff) *gd.soff = isfinite(d) ? -d / (double)gd.V : 0.0;
     }
 }
-
-__global__ void batch_step_increment_kernel(BatchState* st) { st->step += 1; }
 
 // Storage conversion with a per-plane shift: out[i*V + x] = in[i*V + x] - sh[i]
 // (binary16 input: scaled by *scale first).
@@ -345,23 +344,24 @@ __global__ void convert_kernel(const TI* __restrict__ in, TO* __restrict__ out, 
 
 }  // namespace
 
-int launch_batch_reduce(BatchState* state, int max_grids, int grid_stride_bytes, void* stream)
+int launch_batch_reduce(BatchState* state, int K, int max_grids, int grid_stride_bytes,
+                        void* stream)
 {
-    batch_reduce_kernel<<<max_grids, kRedThreads, 0, (cudaStream_t)stream>>>(state,
+    batch_reduce_kernel<<<max_grids, kRedThreads, 0, (cudaStream_t)stream>>>(state, K,
                                                                              grid_stride_bytes);
     return (int)cudaGetLastError();
 }
 
-// One thread per grid of a 64-bit fixed-point batch, after the step and
-// before the step counter moves: the array the grid read this step (parity
+// One thread per grid of a 64-bit fixed-point batch, after step k of a window:
+// the array the grid read this step (parity
 // of its age) is the one its next step writes; set its exponent from the
 // bit length of this step's largest |stored| and reset the bound.
-__global__ void batch_fx_rescale_kernel(const BatchState* st)
+__global__ void batch_fx_rescale_kernel(const BatchState* st, int k)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= st->ngrids) return;
     const BatchGrid<double>& gd = static_cast<const BatchGrid<double>*>(st->grids)[g];
-    const int cur = (int)((st->step - gd.join) & 1);
+    const int cur = (int)((st->step + k - gd.join) & 1);
     const unsigned long long m = *gd.fxmax;
     int sh = 0;
     if (m > (1ull << 54)) sh = (64 - __clzll((long long)m)) - 52;
@@ -369,15 +369,9 @@ __global__ void batch_fx_rescale_kernel(const BatchState* st)
     *gd.fxmax = 0ull;
 }
 
-int launch_batch_fx_rescale(BatchState* state, int max_grids, void* stream)
+int launch_batch_fx_rescale(BatchState* state, int k, int max_grids, void* stream)
 {
-    batch_fx_rescale_kernel<<<(max_grids + 127) / 128, 128, 0, (cudaStream_t)stream>>>(state);
-    return (int)cudaGetLastError();
-}
-
-int launch_batch_increment(BatchState* state, void* stream)
-{
-    batch_step_increment_kernel<<<1, 1, 0, (cudaStream_t)stream>>>(state);
+    batch_fx_rescale_kernel<<<(max_grids + 127) / 128, 128, 0, (cudaStream_t)stream>>>(state, k);
     return (int)cudaGetLastError();
 }
 

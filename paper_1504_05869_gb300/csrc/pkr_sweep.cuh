@@ -394,10 +394,7 @@ __device__ __forceinline__ double pow2(int e)
 }
 
 // The part of a tile step that follows the pull, for velocity group g of G
-// (velocities lo(g) .. lo(g + 1) - 1), as the warp-specialised sweep runs it;
-// tile_step below carries the same operations inline (its binary64 sweep
-// measured 1.9% slower when it called this function instead): the group's
-// share of the density
+// (velocities lo(g) .. lo(g + 1) - 1): the group's share of the density
 // (the G warps of a tile meet at named barrier `bar`, twice in binary64 and
 // once otherwise; every meeting sits outside lane-dependent branches), the
 // relaxation and store of the group's velocities, and, in group 0, the
@@ -440,15 +437,17 @@ __device__ __forceinline__ void group_compute(const TileGrid<T>& tg,
     const int64_t V = tg.V;
     R Phi;
     if constexpr (std::is_same<T, long long>::value) {
-        // fixed point: the density is an exact integer sum
+        // fixed point: the density is an exact integer sum (one group of four
+        // per trip on the x-pairs rows, four in the staged columns)
+        constexpr int FU = VS == 256 ? 4 : 1;
         long long part;
         if constexpr (SPLIT > 0 && SPLIT < n) {
-            part = fx_sum<SPLIT, VS, 1>(sbase);
+            part = fx_sum<SPLIT, VS, FU>(sbase);
             before_tail();
-            part += fx_sum<n - SPLIT, VS, 1>(sbase + SPLIT * VS);
+            part += fx_sum<n - SPLIT, VS, FU>(sbase + SPLIT * VS);
         } else {
             if constexpr (SPLIT >= 0) before_tail();
-            part = fx_sum<n, VS, 1>(sbase);
+            part = fx_sum<n, VS, FU>(sbase);
         }
         if constexpr (G > 1) {
             xacc[g][lane] = part;
@@ -579,204 +578,122 @@ __device__ __forceinline__ void group_compute(const TileGrid<T>& tg,
     }
 }
 
-// One 32-site tile of one grid, executed by the G warps of a tile slot:
-// pull (cp.async), density, relax + store, density output.  On check sweeps
-// the lane's contributions to |dPhi|^2, |Phi|^2, max |dPhi| and sum Phi are
-// added to d2, n2, mx, ms (velocity group 0 only).
-template <class L, typename T, int G, int TILES>
-__device__ __forceinline__ void tile_step(const TileGrid<T>& tg,
-                                          const Coefs<typename AccType<T>::type>& c, int tile,
-                                          int mode, bool zero_in, int lane, int grp, int sub,
-                                          uint32_t sbase, long long (&xacc)[TILES][G][32],
-                                          int (&xexp)[TILES][G][32], double& d2, double& n2,
-                                          double& mx, double& ms, unsigned long long& fxm)
-{
-    using R = typename AccType<T>::type;
-    using ST = Staged<L, T, G, TILES>;
-    constexpr int RC = reach_of<L>();
-    constexpr int W = 2 * RC + 1;
-    constexpr int NC = ncls_of<L>();
-    constexpr int GB = 63 - 53 - ceil_log2(L::Q);
-    static_assert(GB >= 1, "too many velocities for the 64-bit density sum");
-    const T* __restrict__ A = tg.A;
-    T* __restrict__ B = tg.B;
-    const int64_t V = tg.V;
-    const int nx = tg.nx, ny = tg.ny, nz = tg.nz;
-    const int nxy = nx * ny;
-
-    const int64_t s64 = (int64_t)tile * 32 + lane;
-    const bool valid = s64 < V;
-    const int s = valid ? (int)s64 : 0;
-    const int r = (int)((unsigned)s / (unsigned)nx);
-    const int x = s - r * nx;
-    const int z = (int)((unsigned)r / (unsigned)ny);
-    const int y = r - z * ny;
+// The pull of one 32-site tile, per lane: wrapped offsets of the lane's
+// neighbours, and the copy of one velocity's value into the lane's column
+// (dst; zero fill past the grid's end and on the first step).  A lane reads
+// back only what it copied itself, so the copies need no barrier.
+template <class L, typename T>
+struct TilePull {
+    static constexpr int RC = reach_of<L>();
+    static constexpr int W = 2 * RC + 1;
     int xs[W], yo[W], zo[W];
-    if (tg.small) {
-#pragma unroll
-        for (int d = -RC; d <= RC; ++d) {
-            xs[d + RC] = wrap_any(x - d, nx);
-            yo[d + RC] = wrap_any(y - d, ny) * nx;
-            zo[d + RC] = wrap_any(z - d, nz) * nxy;
-        }
-    } else {
-        static_for<0, W>([&](auto DI) {
-            constexpr int d = decltype(DI)::value - RC;
-            xs[d + RC] = wrap_off<d>(x, nx);
-            yo[d + RC] = wrap_off<d>(y, ny) * nx;
-            zo[d + RC] = wrap_off<d>(z, nz) * nxy;
-        });
-    }
-    const int nbytes = (valid && !zero_in) ? (int)sizeof(T) : 0;
-    // the source offset (mass correction) is used by binary32 storage only
-    R Sx = R(0);
-    if (valid) {
-        if constexpr (std::is_same<T, float>::value) Sx = (R)((double)tg.S[s] + tg.soff);
-        else Sx = (R)tg.S[s];
-    }
+    int nbytes;
 
-    static_for<0, G>([&](auto GI) {
-        constexpr int g = decltype(GI)::value;
-        constexpr int lo = ST::lo(g);
-        constexpr int hi = ST::lo(g + 1);
-        constexpr int n = hi - lo;
-        if (grp != g) return;
-        // pull: one asynchronous copy per velocity of this group
-        static_for<lo, hi>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            constexpr int ox = vx_of<L>(i) + RC;
-            constexpr int oy = vy_of<L>(i) + RC;
-            constexpr int oz = vz_of<L>(i) + RC;
-            const T* src = A + ((int64_t)i * V + (zo[oz] + yo[oy] + xs[ox]));
-            cp_async<sizeof(T)>(sbase + (uint32_t)((i - lo) * 32 * sizeof(T)), src, nbytes);
-        });
-        cp_async_wait_all();
-
-        // density (the G warps of a tile meet twice at named barrier 1 + sub;
-        // both barriers sit outside every lane-dependent branch)
-        R Phi;
-        if constexpr (std::is_same<T, long long>::value) {
-            // fixed point: the density is an exact integer sum
-            long long part = fx_sum<n, 256, 4>(sbase);
-            if constexpr (G > 1) {
-                xacc[sub][g][lane] = part;
-                asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "n"(G * 32) : "memory");
-                part = 0;
+    __device__ __forceinline__ void locate(int tile, int64_t V, int nx, int ny, int nz, int small,
+                                           bool zero_in, int lane)
+    {
+        const int nxy = nx * ny;
+        const int64_t s64 = (int64_t)tile * 32 + lane;
+        const bool valid = s64 < V;
+        const int s = valid ? (int)s64 : 0;
+        const int r = (int)((unsigned)s / (unsigned)nx);
+        const int x = s - r * nx;
+        const int z = (int)((unsigned)r / (unsigned)ny);
+        const int y = r - z * ny;
+        if (small) {
 #pragma unroll
-                for (int k = 0; k < G; ++k) part += xacc[sub][k][lane];
-            }
-            Phi = (double)part * pow2(-tg.fr);
-        } else if constexpr (std::is_same<T, double>::value) {
-            int emax = max_exponent<n>(sbase);
-            if constexpr (G > 1) {
-                xexp[sub][g][lane] = emax;
-                asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "n"(G * 32) : "memory");
-#pragma unroll
-                for (int k = 0; k < G; ++k) emax = max(emax, xexp[sub][k][lane]);
-            }
-            const bool plain = plain_path(emax);
-            long long part = plain ? __double_as_longlong(plain_sum<n>(sbase))
-                                   : fixed_sum<GB, n>(sbase, emax);
-            if constexpr (G > 1) {
-                xacc[sub][g][lane] = part;
-                asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "n"(G * 32) : "memory");
-                if (plain) {
-                    double t = 0.0;
-#pragma unroll
-                    for (int k = 0; k < G; ++k) t += __longlong_as_double(xacc[sub][k][lane]);
-                    Phi = t;
-                } else {
-                    long long t = 0;
-#pragma unroll
-                    for (int k = 0; k < G; ++k) t += xacc[sub][k][lane];
-                    Phi = fixed_value<GB>(t, emax);
-                }
-            } else {
-                Phi = plain ? __longlong_as_double(part) : fixed_value<GB>(part, emax);
+            for (int d = -RC; d <= RC; ++d) {
+                xs[d + RC] = wrap_any(x - d, nx);
+                yo[d + RC] = wrap_any(y - d, ny) * nx;
+                zo[d + RC] = wrap_any(z - d, nz) * nxy;
             }
         } else {
-            float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll 2
-            for (int k = 0; k + 3 < n; k += 4) {
-                s0 += lds_f32(sbase + (k + 0) * 128);
-                s1 += lds_f32(sbase + (k + 1) * 128);
-                s2 += lds_f32(sbase + (k + 2) * 128);
-                s3 += lds_f32(sbase + (k + 3) * 128);
-            }
-#pragma unroll
-            for (int k = n - n % 4; k < n; ++k) s0 += lds_f32(sbase + k * 128);
-            float part = (s0 + s1) + (s2 + s3);
-            if constexpr (G > 1) {
-                // binary32 partials meet in group order (fixed, deterministic)
-                xacc[sub][g][lane] = (long long)__float_as_int(part);
-                asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "n"(G * 32) : "memory");
-                part = 0.f;
-#pragma unroll
-                for (int k = 0; k < G; ++k) part += __int_as_float((int)xacc[sub][k][lane]);
-            }
-            Phi = part;
-        }
-
-        // relax and store this group's velocities, one symmetry class at a
-        // time (velocities of a class are contiguous and share phi_c, chi_c)
-        if (valid) {
-            static_for<0, NC>([&](auto CI) {
-                constexpr int cl = decltype(CI)::value;
-                constexpr int cb = cls_begin<L>(cl), ce = cls_begin<L>(cl + 1);
-                constexpr int i0 = cb > lo ? cb : lo;
-                constexpr int i1 = ce < hi ? ce : hi;
-                if constexpr (i0 < i1 && std::is_same<T, long long>::value) {
-                    const double e = fma(c.wphi[cl], Phi, c.chi[cl] * Sx);
-                    const long long ei = __double2ll_rn(e * pow2(tg.fw));
-                    // the written array's scale is 2^-k that of the read one (k >= 0,
-                    // the rescale only lowers it): fold 2^-k into the coefficient
-                    const int k = tg.fr - tg.fw;
-                    const long long cw = k == 0 ? tg.cfx : ((tg.cfx >> (k - 1)) + 1) >> 1;
-                    T* dst = B + ((int64_t)i0 * V + s);
-#pragma unroll 2
-                    for (int i = i0; i < i1; ++i) {
-                        const long long p = fx_mul(lds_s64(sbase + (i - lo) * 256), cw) + ei;
-                        fxm |= (unsigned long long)(p ^ (p >> 63));
-                        store_stream(dst, (T)p);
-                        dst += V;
-                    }
-                } else if constexpr (i0 < i1) {
-                    const R e = fma(c.wphi[cl], Phi, c.chi[cl] * Sx);
-                    T* dst = B + ((int64_t)i0 * V + s);
-                    int i = i0;
-                    for (; i + 3 < i1; i += 4) {
-                        const R g0 = lds_val<T>(sbase + (i + 0 - lo) * 32 * sizeof(T));
-                        const R g1 = lds_val<T>(sbase + (i + 1 - lo) * 32 * sizeof(T));
-                        const R g2 = lds_val<T>(sbase + (i + 2 - lo) * 32 * sizeof(T));
-                        const R g3 = lds_val<T>(sbase + (i + 3 - lo) * 32 * sizeof(T));
-                        store_stream(dst, (T)fma(c.om1, g0, e));
-                        store_stream(dst + V, (T)fma(c.om1, g1, e));
-                        store_stream(dst + 2 * V, (T)fma(c.om1, g2, e));
-                        store_stream(dst + 3 * V, (T)fma(c.om1, g3, e));
-                        dst += 4 * V;
-                    }
-                    for (; i < i1; ++i) {
-                        const R gi = lds_val<T>(sbase + (i - lo) * 32 * sizeof(T));
-                        store_stream(dst, (T)fma(c.om1, gi, e));
-                        dst += V;
-                    }
-                }
+            static_for<0, W>([&](auto DI) {
+                constexpr int d = decltype(DI)::value - RC;
+                xs[d + RC] = wrap_off<d>(x, nx);
+                yo[d + RC] = wrap_off<d>(y, ny) * nx;
+                zo[d + RC] = wrap_off<d>(z, nz) * nxy;
             });
         }
-        // density output and residual contributions (one group per tile)
-        if (g == 0 && mode != kPlain && valid) {
-            const double ph = (double)Phi;
-            if (mode == kCheck) {
-                const double d = ph - tg.Phi[s];
-                d2 += d * d;
-                n2 += ph * ph;
-                mx = fmax(mx, fabs(d));
-                ms += ph;
-            }
-            tg.Phi[s] = ph;
-        }
-    });
-    __syncwarp();
+        nbytes = (valid && !zero_in) ? (int)sizeof(T) : 0;
+    }
+    template <int i>
+    __device__ __forceinline__ void pull(const T* __restrict__ A, int64_t V, uint32_t dst) const
+    {
+        const T* src = A + ((int64_t)i * V + (zo[vz_of<L>(i) + RC] + yo[vy_of<L>(i) + RC] +
+                                              xs[vx_of<L>(i) + RC]));
+        cp_async<sizeof(T)>(dst, src, nbytes);
+    }
+};
+
+// First velocity of the last symmetry class that velocities lo .. hi - 1 hold.
+template <class L>
+__host__ __device__ constexpr int tail_begin(int lo, int hi)
+{
+    const int b = cls_begin<L>(cls_of<L>(hi - 1));
+    return b > lo ? b : lo;
+}
+
+// (small sets: D3Q19 at 256^3 17.9 GLUPS with early refill, 18.1 without)
+template <class L, typename T>
+struct EarlyRefill {
+    static constexpr bool value = L::Q > 64 && std::is_same<T, double>::value;
+};
+// One tile of velocity group g.  In binary64 its copies are in flight already,
+// and class by class as it is relaxed the copies of the warp's next tile
+// (`refill(I)` copies velocity I of it) are started, so the pull of a tile
+// overlaps the computation of the one before; each class is a copy group of
+// its own, so a tile starts once every class but its last (refilled last) has
+// landed, as in the x-pairs sweep.  The other storages copy a tile at its
+// start.  GLUPS on 173 x 141 x
+// 100, D3Q111, 2 groups x 2 tiles, early refill against copies at the start:
+// binary64 2.64 / 2.41, fixed point 2.88 / 2.91, binary32 5.15 / 5.56.
+template <class L, typename T, int G, int g, class Refill>
+__device__ __forceinline__ void tile_compute(const TileGrid<T>& tg,
+                                             const Coefs<typename AccType<T>::type>& c, int mode,
+                                             bool valid, int s, typename AccType<T>::type Sx,
+                                             int lane, uint32_t sbase, int bar,
+                                             long long (&xacc)[G][32], int (&xexp)[G][32],
+                                             double& d2, double& n2, double& mx, double& ms,
+                                             unsigned long long& fxm, bool more,
+                                             const Refill& refill)
+{
+    constexpr int lo = g * L::Q / G, hi = (g + 1) * L::Q / G;
+    constexpr int VS = 32 * (int)sizeof(T);
+    constexpr int tb = tail_begin<L>(lo, hi);
+    if constexpr (EarlyRefill<L, T>::value) {
+        cp_async_wait_all_but_last();
+        group_compute<L, T, G, g, VS, tb - lo>(
+            tg, c, mode, valid, s, Sx, lane, sbase, bar, xacc, xexp, d2, n2, mx, ms, fxm,
+            [&](auto CI) {
+                constexpr int cl = decltype(CI)::value;
+                constexpr int cb = cls_begin<L>(cl), ce = cls_begin<L>(cl + 1);
+                if (more) {
+                    static_for<(cb > lo ? cb : lo), (ce < hi ? ce : hi)>(refill);
+                    cp_async_commit();
+                }
+            },
+            [&]() { cp_async_wait_committed(); });
+    } else {
+        static_for<lo, hi>(refill);
+        cp_async_wait_all();
+        group_compute<L, T, G, g, VS>(tg, c, mode, valid, s, Sx, lane, sbase, bar, xacc, xexp, d2,
+                                      n2, mx, ms, fxm);
+    }
+}
+
+// The first tile's copies, in the groups tile_compute waits for.
+template <class L, typename T, int G, int g, class Refill>
+__device__ __forceinline__ void tile_first(const Refill& refill)
+{
+    constexpr int lo = g * L::Q / G, hi = (g + 1) * L::Q / G;
+    constexpr int tb = tail_begin<L>(lo, hi);
+    if constexpr (EarlyRefill<L, T>::value) {
+        static_for<lo, tb>(refill);
+        cp_async_commit();
+        static_for<tb, hi>(refill);
+        cp_async_commit();
+    }
 }
 
 template <class L, typename T, int G_, int TILES_>
@@ -811,9 +728,43 @@ sweep_staged_kernel(const SweepArgs a, const Coefs<typename AccType<T>::type> c)
     unsigned long long fxm = 0ull;
     const int nt = gridDim.x * TILES;
     int par = 0;
-    for (int tile = blockIdx.x * TILES + sub; tile < a.ntiles; tile += nt, par ^= 1)
-        tile_step<L, T, G, TILES>(tg, c, tile, a.mode, a.zero_in != 0, lane, grp, sub, sbase,
-                                  xacc[par], xexp, rd2, rn2, rmx, rms, fxm);
+    static_for<0, G>([&](auto GI) {
+        constexpr int g = decltype(GI)::value;
+        if (grp != g) return;
+        using R = typename AccType<T>::type;
+        TilePull<L, T> next;
+        auto refill = [&](auto I) {
+            constexpr int i = decltype(I)::value;
+            next.template pull<i>(tg.A, tg.V, sbase + (uint32_t)((i - ST::lo(g)) * 32 * sizeof(T)));
+        };
+        int tile = blockIdx.x * TILES + sub;
+        if (EarlyRefill<L, T>::value && tile < a.ntiles) {
+            next.locate(tile, tg.V, tg.nx, tg.ny, tg.nz, tg.small, a.zero_in != 0, lane);
+            tile_first<L, T, G, g>(refill);
+        }
+        for (; tile < a.ntiles; tile += nt, par ^= 1) {
+            const int64_t s64 = (int64_t)tile * 32 + lane;
+            const bool valid = s64 < tg.V;
+            // the source offset (mass correction) is used by binary32 storage only
+            R Sx = R(0);
+            if (valid) {
+                if constexpr (std::is_same<T, float>::value)
+                    Sx = (R)((double)tg.S[s64] + tg.soff);
+                else Sx = (R)tg.S[s64];
+            }
+            const bool more = tile + nt < a.ntiles;
+            if constexpr (EarlyRefill<L, T>::value) {
+                if (more)
+                    next.locate(tile + nt, tg.V, tg.nx, tg.ny, tg.nz, tg.small, a.zero_in != 0,
+                                lane);
+            } else {
+                next.locate(tile, tg.V, tg.nx, tg.ny, tg.nz, tg.small, a.zero_in != 0, lane);
+            }
+            tile_compute<L, T, G, g>(tg, c, a.mode, valid, (int)s64, Sx, lane, sbase, 1 + sub,
+                                     xacc[par][sub], xexp[sub], rd2, rn2, rmx, rms, fxm, more,
+                                     refill);
+        }
+    });
     if constexpr (std::is_same<T, long long>::value) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -858,17 +809,21 @@ sweep_staged_kernel(const SweepArgs a, const Coefs<typename AccType<T>::type> c)
 // ---------------------------------------------------------------------------
 // Batch sweep: one persistent launch advances every live grid of a batch by
 // one step.  Batch-wide tile t belongs to the grid whose tile_begin is the
-// largest one <= t (binary search over the descriptors).  A grid's age (steps
-// since it joined) picks its buffers and its own residual schedule: it writes
-// Phi when (age + 2) % K == 0 and checks when (age + 1) % K == 0 (age >= 1),
-// so a grid's trajectory and stopping step do not depend on what else is in
-// the batch.  On check steps each tile leaves its four partial sums in
-// tile_partials (with the sum of Phi); pkr_batch_reduce sums them per grid in
-// a fixed order.
+// largest one <= t (binary search over the descriptors for a warp's first
+// tile, a walk from there on).  A grid's age (steps since it joined) picks its
+// buffers; it joins at a window's start, so the position k of the step in its
+// window of K steps, the same for every grid, gives the residual schedule of
+// its own age: Phi is written when (age + 2) % K == 0 and checked when
+// (age + 1) % K == 0 (age >= 1), and a grid's trajectory and stopping step do
+// not depend on what else is in the batch.  The host passes these as `phase`:
+// as three 64-bit remainders per tile and warp they cost as much as a third of
+// a binary32 tile.  On check steps each tile leaves its four partial sums in
+// tile_partials (with the sum of Phi); batch_reduce_kernel sums them per grid
+// in a fixed order.
 // ---------------------------------------------------------------------------
 template <class L, typename T, int G_, int TILES_>
 __global__ void __launch_bounds__(G_ * TILES_ * 32)
-sweep_batch_kernel(BatchState* st, int K)
+sweep_batch_kernel(BatchState* st, int k, int phase)
 {
     using R = typename AccType<T>::type;
     constexpr int G = G_;
@@ -887,36 +842,40 @@ sweep_batch_kernel(BatchState* st, int K)
     const BatchGrid<R>* grids = static_cast<const BatchGrid<R>*>(st->grids);
     const int ngrids = st->ngrids;
     const int ntiles = st->ntiles;
-    const long long step = st->step;
+    const long long step = st->step + k;
     double* tpart = st->tile_partials;
 
+    constexpr bool fx = std::is_same<T, long long>::value;
     const int nt = gridDim.x * TILES;
     int par = 0;
-    for (int tile = blockIdx.x * TILES + sub; tile < ntiles; tile += nt, par ^= 1) {
+    // index of the grid that tile t belongs to
+    auto grid_of = [&](int t) {
         int lo = 0, hi = ngrids - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (grids[mid].tile_begin <= tile) lo = mid;
+            if (grids[mid].tile_begin <= t) lo = mid;
             else hi = mid - 1;
         }
-        const BatchGrid<R>& gd = grids[lo];
-        const long long age = step - gd.join;
+        return lo;
+    };
+    auto mode_of = [&](long long age) {
+        if (age >= 1 && (phase & kPhaseCheck)) return (int)kCheck;
+        return age == 0 || (phase & kPhaseWrite) ? (int)kWritePhi : (int)kPlain;
+    };
+    // binary32: the step after a check removes the mass that check measured
+    auto soff_of = [&](const BatchGrid<R>& gd, long long age) {
+        return gd.soff && age >= 1 && (phase & kPhaseFirst) ? *gd.soff : 0.0;
+    };
+    auto state_of = [&](const BatchGrid<R>& gd, long long age, double soff) {
         const int cur = (int)(age & 1);
-        const bool zero_in = (age == 0);
-        int mode = kPlain;
-        if (age >= 1 && (age + 1) % K == 0) mode = kCheck;
-        else if (zero_in || (age + 2) % K == 0) mode = kWritePhi;
-        constexpr bool fx = std::is_same<T, long long>::value;
-        // binary32: the step after a check removes the mass that check measured
-        const double soff = (gd.soff && age >= 1 && age % K == 0) ? *gd.soff : 0.0;
-        const TileGrid<T> tg{static_cast<const T*>(gd.pop[cur]), static_cast<T*>(gd.pop[cur ^ 1]),
-                             static_cast<const typename SrcType<T>::type*>(gd.S), gd.Phi, gd.V,
-                             gd.nx, gd.ny, gd.nz, gd.small, soff, fx ? gd.fxF[cur] : 0,
-                             fx ? gd.fxF[cur ^ 1] : 0, fx ? gd.cfx : 0};
-        double d2 = 0.0, n2 = 0.0, mx = 0.0, ms = 0.0;
-        unsigned long long fxm = 0ull;
-        tile_step<L, T, G, TILES>(tg, gd.c, tile - gd.tile_begin, mode, zero_in, lane, grp, sub,
-                                  sbase, xacc[par], xexp, d2, n2, mx, ms, fxm);
+        return TileGrid<T>{static_cast<const T*>(gd.pop[cur]), static_cast<T*>(gd.pop[cur ^ 1]),
+                           static_cast<const typename SrcType<T>::type*>(gd.S), gd.Phi, gd.V,
+                           gd.nx, gd.ny, gd.nz, gd.small, soff, fx ? gd.fxF[cur] : 0,
+                           fx ? gd.fxF[cur ^ 1] : 0, fx ? gd.cfx : 0};
+    };
+    // a tile's magnitude bound and residual terms
+    auto finish = [&](const BatchGrid<R>& gd, int tile, int mode, double d2, double n2, double mx,
+                      double ms, unsigned long long fxm) {
         if constexpr (fx) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) fxm |= __shfl_down_sync(0xffffffffu, fxm, o);
@@ -937,16 +896,67 @@ sweep_batch_kernel(BatchState* st, int K)
                 tpart[4 * (int64_t)tile + 3] = ms;
             }
         }
-    }
+    };
+    static_for<0, G>([&](auto GI) {
+        constexpr int g = decltype(GI)::value;
+        if (grp != g) return;
+        int tile = blockIdx.x * TILES + sub;
+        if (tile >= ntiles) return;
+        int gi = grid_of(tile);
+        TilePull<L, T> next;
+        const T* A = nullptr;
+        int64_t V = 0;
+        // tile t of grid gi, whose copies come next
+        auto locate = [&](int t) {
+            const BatchGrid<R>& gd = grids[gi];
+            const long long age = step - gd.join;
+            A = static_cast<const T*>(gd.pop[age & 1]);
+            V = gd.V;
+            next.locate(t - gd.tile_begin, V, gd.nx, gd.ny, gd.nz, gd.small, age == 0, lane);
+        };
+        auto refill = [&](auto I) {
+            constexpr int i = decltype(I)::value;
+            next.template pull<i>(A, V, sbase + (uint32_t)((i - ST::lo(g)) * 32 * sizeof(T)));
+        };
+        if constexpr (EarlyRefill<L, T>::value) locate(tile);
+        tile_first<L, T, G, g>(refill);
+        for (; tile < ntiles; tile += nt, par ^= 1) {
+            const BatchGrid<R>& gd = grids[gi];
+            const long long age = step - gd.join;
+            const int mode = mode_of(age);
+            const TileGrid<T> tg = state_of(gd, age, soff_of(gd, age));
+            const int64_t s64 = (int64_t)(tile - gd.tile_begin) * 32 + lane;
+            const bool valid = s64 < tg.V;
+            R Sx = R(0);
+            if (valid) {
+                if constexpr (std::is_same<T, float>::value)
+                    Sx = (R)((double)tg.S[s64] + tg.soff);
+                else Sx = (R)tg.S[s64];
+            }
+            const bool more = tile + nt < ntiles;
+            if constexpr (!EarlyRefill<L, T>::value) locate(tile);
+            // the next tile's grid is this one or a later one
+            if (more)
+                while (gi + 1 < ngrids && grids[gi + 1].tile_begin <= tile + nt) ++gi;
+            if constexpr (EarlyRefill<L, T>::value) {
+                if (more) locate(tile + nt);
+            }
+            double d2 = 0.0, n2 = 0.0, mx = 0.0, ms = 0.0;
+            unsigned long long fxm = 0ull;
+            tile_compute<L, T, G, g>(tg, gd.c, mode, valid, (int)s64, Sx, lane, sbase, 1 + sub,
+                                     xacc[par][sub], xexp[sub], d2, n2, mx, ms, fxm, more, refill);
+            finish(gd, tile, mode, d2, n2, mx, ms, fxm);
+        }
+    });
 }
 
 template <class L, typename T, int K>
-int launch_batch_variant(BatchState* st, int check_every, int grid, void* stream)
+int launch_batch_variant(BatchState* st, int k, int phase, int grid, void* stream)
 {
     constexpr Geo geo = Variants<L>::at(K);
     using ST = Staged<L, T, geo.G, geo.TILES>;
     sweep_batch_kernel<L, T, geo.G, geo.TILES><<<grid, ST::WARPS * 32, ST::smem_bytes(),
-                                                 (cudaStream_t)stream>>>(st, check_every);
+                                                 (cudaStream_t)stream>>>(st, k, phase);
     return (int)cudaGetLastError();
 }
 
@@ -963,12 +973,12 @@ int batch_occupancy_variant(int* blocks)
 }
 
 template <class L, typename T>
-int launch_batch_t(int variant, BatchState* st, int check_every, int grid, void* stream)
+int launch_batch_t(int variant, BatchState* st, int k, int phase, int grid, void* stream)
 {
     int rc = (int)cudaErrorInvalidValue;
     static_for<0, Variants<L>::N>([&](auto K) {
         if (variant == decltype(K)::value)
-            rc = launch_batch_variant<L, T, decltype(K)::value>(st, check_every, grid, stream);
+            rc = launch_batch_variant<L, T, decltype(K)::value>(st, k, phase, grid, stream);
     });
     return rc;
 }
@@ -1574,9 +1584,9 @@ int batch_variant_count_t() { return Variants<L>::N; }
                                    const int*);                                                 \
     template int resident_form<L>(int64_t, int, int, int);                                   \
     template int launch_resident<L>(int, const CoopArgs&, const Coefs<double>&, void*);      \
-    template int launch_batch_t<L, double>(int, BatchState*, int, int, void*);               \
-    template int launch_batch_t<L, float>(int, BatchState*, int, int, void*);                \
-    template int launch_batch_t<L, long long>(int, BatchState*, int, int, void*);            \
+    template int launch_batch_t<L, double>(int, BatchState*, int, int, int, void*);         \
+    template int launch_batch_t<L, float>(int, BatchState*, int, int, int, void*);          \
+    template int launch_batch_t<L, long long>(int, BatchState*, int, int, int, void*);      \
     template int batch_occupancy_t<L, double>(int, int*);                                    \
     template int batch_occupancy_t<L, long long>(int, int*);                                 \
     template int batch_occupancy_t<L, float>(int, int*);

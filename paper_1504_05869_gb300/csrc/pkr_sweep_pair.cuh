@@ -109,14 +109,6 @@ struct PairFill {
     }
 };
 
-// First velocity of the last symmetry class that velocities lo .. hi - 1 hold.
-template <class L>
-__host__ __device__ constexpr int tail_begin(int lo, int hi)
-{
-    const int b = cls_begin<L>(cls_of<L>(hi - 1));
-    return b > lo ? b : lo;
-}
-
 template <class L, typename T, int G, bool EARLY>
 __global__ void __launch_bounds__(64 * G)
 sweep_pair_kernel(const SweepArgs a, const Coefs<typename AccType<T>::type> c)
