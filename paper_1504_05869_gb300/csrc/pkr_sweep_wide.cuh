@@ -23,7 +23,11 @@ struct Wide {
     static constexpr int HL = (reach_of<L>() + 3) / 4 * 4;   // halo values per side
     static constexpr int RL = 64 + 2 * HL;
     static constexpr int ROWB = RL * 4;
-    static constexpr int PAIRS = 3;                          // 64-site pairs per block
+    // 64-site pairs per block: one block of 12 warps per SM.  GB/s at 192^3 and
+    // 256 x 256 x 160, D3Q111: 6 pairs 5905 / 5807, 4 pairs 5898 / 5748 (8
+    // warps), 3 pairs x 2 blocks 5713 / 5697, 2 pairs x 3 blocks 4877 / 4875,
+    // 7 pairs 4631 / 4570 (too little of the SM left for L1).
+    static constexpr int PAIRS = L::Q > 111 ? 3 : 6;
     static constexpr int THREADS = PAIRS * G * 32;
     static constexpr size_t smem_bytes() { return (size_t)PAIRS * Q * ROWB; }
 };
@@ -44,7 +48,7 @@ __device__ __forceinline__ f32x2 row_pair(uint32_t addr)
 }
 
 template <class L>
-__global__ void __launch_bounds__(Wide<L>::THREADS, 2)
+__global__ void __launch_bounds__(Wide<L>::THREADS, 1)
 sweep_wide_kernel(const SweepArgs a, const Coefs<float> c)
 {
     if (a.stop != nullptr && *a.stop != 0) return;   // the run stopped before this step
