@@ -201,8 +201,8 @@ struct pkr_plan {
     double* partials;
     double* scal;   // [0] source mean, [1..4] residual out, [5] mean of an imported Phi
     int* flag;
-    double* host;   // pinned: [0] mean, [1..4] residual, [5] import mean, [6] flag (int),
-                    // [7] binary16 overflow flag (int)
+    double host[6]; // read back: [0] mean, [1..4] residual, [5] import mean
+    void* slab;     // device block of S, Phi (or the stencil's arrays) and the scratch below
     bool stencil;          // omega = 1, binary64: the state is Phi alone (scalar stencil)
     int planes;            // stencil mode: z chunk of the plane form, 0: one thread per site
     double* Ps[2];         // stencil mode: Phi ping-pong
@@ -218,8 +218,8 @@ struct pkr_plan {
     // device-side stopping (binary64 runs that check every step): a captured
     // graph of kGraphSteps check steps, each followed by the stopping rule on
     // the device; steps after a stop return at once (SweepArgs::stop)
-    RunCtl* ctl;           // device state of the rule
-    RunCtl* hctl;          // pinned host copy
+    RunCtl* ctl;           // device state of the rule (the step barrier's counter follows)
+    RunCtl hctl;           // host copy
     cudaGraphExec_t gexec; // the captured steps (nullptr: none yet)
     cudaStream_t cap;      // stream the graph is captured on
     int gcur, gkind, gj;   // array parity and tol kind the graph was captured for;
@@ -434,21 +434,9 @@ constexpr int kStallChecks = 4;
 // arrays are back at the same parity after a full replay).
 constexpr int kGraphSteps = 64;
 
-// Device and host copies of the rule's state; the step barrier's counter
-// follows the device one.
+// Device bytes of the rule's state and, at byte 64, the step barrier's counter.
 constexpr size_t kCtlBytes = 128;
-int alloc_ctl(pkr_plan* P)
-{
-    static_assert(sizeof(RunCtl) <= 64, "the counter sits at byte 64");
-    if (cudaMalloc((void**)&P->ctl, kCtlBytes) != cudaSuccess ||
-        cudaMallocHost((void**)&P->hctl, sizeof(RunCtl)) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(P->ctl);
-        P->ctl = nullptr;
-        return PKR_ENOMEM;
-    }
-    return PKR_OK;
-}
+static_assert(sizeof(RunCtl) <= 64, "the counter sits at byte 64");
 
 // Steps per launch of a resident run: tens of milliseconds at most.
 constexpr int64_t kResidentSteps = 8192;
@@ -516,10 +504,9 @@ int launch_resident_steps(pkr_plan* P, int form, int nsteps, double tol, int kin
     return rc == 0 ? PKR_OK : PKR_ECUDA;
 }
 
-// Memory of a resident run (its rule's state, and the sweep's third array).
+// Memory of a resident run: the sweep's third array.
 bool resident_ready(pkr_plan* P, int form)
 {
-    if (!P->ctl && alloc_ctl(P) != PKR_OK) return false;
     if (form == 3 && !P->pop3 &&
         cudaMalloc(&P->pop3, (size_t)P->lat.Q * (size_t)P->V * 8 + 16) != cudaSuccess) {
         cudaGetLastError();
@@ -555,10 +542,6 @@ void resident_advance(pkr_plan* P, int form, int64_t ran)
 // afterwards: capturing runs nothing.  On failure the caller steps on the host.
 int capture_steps(pkr_plan* P, double tol, int tol_kind)
 {
-    if (!P->ctl) {
-        const int rc = alloc_ctl(P);
-        if (rc != PKR_OK) return rc;
-    }
     if (!P->cap && cudaStreamCreateWithFlags(&P->cap, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         P->cap = nullptr;
@@ -809,29 +792,43 @@ int plan_create(const pkr_problem* p, void* stream, pkr_plan** out, bool spare)
         delete P;
         return PKR_ENOMEM;
     }
-    const size_t nscratch = (size_t)4 * kMaxGridBlocks;
-    bool ok = (P->stencil
-                   ? (cudaMalloc((void**)&P->Ps[0], (size_t)P->V * 8) == cudaSuccess &&
-                      cudaMalloc((void**)&P->Ps[1], (size_t)P->V * 8) == cudaSuccess &&
-                      cudaMalloc((void**)&P->St, (size_t)P->V * 8) == cudaSuccess)
-                   : (cudaMalloc(&P->pop[0], popb) == cudaSuccess &&
-                      (!spare || cudaMalloc(&P->pop[1], popb) == cudaSuccess))) &&
-              cudaMalloc(&P->S, (size_t)P->V * source_bytes(p->precision)) == cudaSuccess &&
-              cudaMalloc((void**)&P->h16sc, 2 * sizeof(float)) == cudaSuccess &&
-              cudaMalloc((void**)&P->h16max, sizeof(unsigned int)) == cudaSuccess &&
-              cudaMalloc((void**)&P->h16of, sizeof(int)) == cudaSuccess &&
-              cudaMalloc((void**)&P->fxF, 2 * sizeof(int)) == cudaSuccess &&
-              cudaMalloc((void**)&P->fxmax, sizeof(unsigned long long)) == cudaSuccess &&
-              (P->stencil || cudaMalloc((void**)&P->Phi, (size_t)P->V * 8) == cudaSuccess) &&
-              cudaMalloc((void**)&P->partials, nscratch * 8) == cudaSuccess &&
-              cudaMalloc((void**)&P->scal, 8 * 8) == cudaSuccess &&
-              cudaMalloc((void**)&P->flag, sizeof(int)) == cudaSuccess &&
-              cudaMallocHost((void**)&P->host, 8 * 8) == cudaSuccess;
-    if (!ok) {
+    // One block for S, Phi (stencil: S, both Phi arrays and St) and the
+    // scratch, and the populations each by itself (a ladder frees and adds
+    // them).  Fourteen blocks and two pinned ones cost a 64-site solve 0.3 of
+    // its 3.4 ms.
+    const size_t vb = ((size_t)P->V * 8 + 255) / 256 * 256;
+    const size_t sb = ((size_t)P->V * source_bytes(p->precision) + 255) / 256 * 256;
+    const size_t pb = (size_t)4 * kMaxGridBlocks * 8;
+    if ((!P->stencil && (cudaMalloc(&P->pop[0], popb) != cudaSuccess ||
+                         (spare && cudaMalloc(&P->pop[1], popb) != cudaSuccess))) ||
+        cudaMalloc(&P->slab, (P->stencil ? 3 : 1) * vb + sb + pb + 512) != cudaSuccess) {
         cudaGetLastError();
         pkr_plan_destroy(P);
         return PKR_ENOMEM;
     }
+    unsigned char* at = static_cast<unsigned char*>(P->slab);
+    auto take = [&](size_t bytes) {
+        void* p = at;
+        at += bytes;
+        return p;
+    };
+    P->S = take(sb);
+    if (P->stencil) {
+        P->Ps[0] = static_cast<double*>(take(vb));
+        P->Ps[1] = static_cast<double*>(take(vb));
+        P->St = static_cast<double*>(take(vb));
+    } else {
+        P->Phi = static_cast<double*>(take(vb));
+    }
+    P->partials = static_cast<double*>(take(pb));
+    P->scal = static_cast<double*>(take(64));
+    P->flag = static_cast<int*>(take(64));      // right after scal: read back together
+    P->ctl = static_cast<RunCtl*>(take(kCtlBytes));
+    P->fxmax = static_cast<unsigned long long*>(take(8));
+    P->fxF = static_cast<int*>(take(8));
+    P->h16sc = static_cast<float*>(take(8));
+    P->h16max = static_cast<unsigned int*>(take(4));
+    P->h16of = static_cast<int*>(take(4));
     if (P->stencil) P->Phi = P->Ps[0];
     *out = P;
     return PKR_OK;
@@ -872,27 +869,12 @@ int pkr_plan_create(const pkr_problem* p, void* stream, pkr_plan** out)
 int pkr_plan_destroy(pkr_plan* P)
 {
     if (!P) return PKR_OK;
-    if (P->stream || P->pop[0] || P->Ps[0]) cudaStreamSynchronize(P->stream);
+    if (P->stream || P->pop[0] || P->slab) cudaStreamSynchronize(P->stream);
     cudaFree(P->pop[0]);
     cudaFree(P->pop[1]);
     cudaFree(P->pop3);
-    cudaFree(P->Ps[0]);
-    cudaFree(P->Ps[1]);
-    cudaFree(P->St);
-    cudaFree(P->S);
-    if (!P->stencil) cudaFree(P->Phi);
-    cudaFree(P->partials);
-    cudaFree(P->scal);
-    cudaFree(P->flag);
-    cudaFree(P->h16sc);
-    cudaFree(P->h16max);
-    cudaFree(P->h16of);
-    cudaFree(P->fxF);
-    cudaFree(P->fxmax);
-    if (P->host) cudaFreeHost(P->host);
+    cudaFree(P->slab);
     if (P->gexec) cudaGraphExecDestroy(P->gexec);
-    cudaFree(P->ctl);
-    if (P->hctl) cudaFreeHost(P->hctl);
     if (P->cap) cudaStreamDestroy(P->cap);
     delete P;
     return PKR_OK;
@@ -929,16 +911,16 @@ int load_source(pkr_plan* P, const double* rho, int rho_on_host, bool first_step
         if (launch_absmax_f32(static_cast<const float*>(P->S), P->V, P->h16max, P->stream) != 0)
             return PKR_ECUDA;
     }
-    PKR_CK(cudaMemcpyAsync(P->host, P->scal, 8, cudaMemcpyDeviceToHost, P->stream));
-    PKR_CK(cudaMemcpyAsync(P->host + 6, P->flag, sizeof(int), cudaMemcpyDeviceToHost, P->stream));
+    double back[9];   // scal, then the flag
+    PKR_CK(cudaMemcpyAsync(back, P->scal, sizeof(back), cudaMemcpyDeviceToHost, P->stream));
     PKR_CK(cudaStreamSynchronize(P->stream));
     int bad = 0;
-    std::memcpy(&bad, P->host + 6, sizeof(int));
+    std::memcpy(&bad, back + 8, sizeof(int));
     if (bad) {
         P->loaded = false;
         return PKR_EINVAL;
     }
-    P->rho_mean = P->host[0];
+    P->rho_mean = back[0];
     if (P->prob.precision == PKR_FX64) {
         // exponent of the first write (the step from zero stores chi_i S):
         // its largest value lands near 2^52, leaving room to grow before the
@@ -1158,10 +1140,10 @@ int pkr_plan_run(pkr_plan* P, int64_t steps, double tol, int tol_kind, int check
         // small grids: all steps in a few resident launches
         const int form = resident_of(P);
         if (form > 0 && resident_ready(P, form)) {
-            *P->hctl = RunCtl{0, PKR_OK, -1, 0, INFINITY, P->last_residual};
+            P->hctl = RunCtl{0, PKR_OK, -1, 0, INFINITY, P->last_residual};
             while (done < steps && !stopped) {
                 const int64_t n = steps - done < kResidentSteps ? steps - done : kResidentSteps;
-                PKR_CK(cudaMemcpyAsync(P->ctl, P->hctl, sizeof(RunCtl), cudaMemcpyHostToDevice,
+                PKR_CK(cudaMemcpyAsync(P->ctl, &P->hctl, sizeof(RunCtl), cudaMemcpyHostToDevice,
                                        P->stream));
                 PKR_CK(cudaMemsetAsync(reinterpret_cast<char*>(P->ctl) + 64, 0,
                                        sizeof(unsigned int), P->stream));
@@ -1171,10 +1153,10 @@ int pkr_plan_run(pkr_plan* P, int64_t steps, double tol, int tol_kind, int check
                     P->resident = 0;
                     break;
                 }
-                PKR_CK(cudaMemcpyAsync(P->hctl, P->ctl, sizeof(RunCtl), cudaMemcpyDeviceToHost,
+                PKR_CK(cudaMemcpyAsync(&P->hctl, P->ctl, sizeof(RunCtl), cudaMemcpyDeviceToHost,
                                        P->stream));
                 PKR_CK(cudaStreamSynchronize(P->stream));
-                const RunCtl c = *P->hctl;
+                const RunCtl c = P->hctl;
                 if (c.status == PKR_ECUDA) return PKR_ECUDA;
                 resident_advance(P, form, (int64_t)c.done_at + 1);
                 done += (int64_t)c.done_at + 1;
@@ -1190,15 +1172,15 @@ int pkr_plan_run(pkr_plan* P, int64_t steps, double tol, int tol_kind, int check
         } else if (!P->gexec || P->gcur != P->cur || P->gtol != tol || P->gkind != tol_kind)
             ok = capture_steps(P, tol, tol_kind) == PKR_OK;
         if (ok) {
-            *P->hctl = RunCtl{0, PKR_OK, -1, 0, INFINITY, P->last_residual};
-            PKR_CK(cudaMemcpyAsync(P->ctl, P->hctl, sizeof(RunCtl), cudaMemcpyHostToDevice,
+            P->hctl = RunCtl{0, PKR_OK, -1, 0, INFINITY, P->last_residual};
+            PKR_CK(cudaMemcpyAsync(P->ctl, &P->hctl, sizeof(RunCtl), cudaMemcpyHostToDevice,
                                    P->stream));
             while (steps - done >= kGraphSteps) {
                 PKR_CK(cudaGraphLaunch(P->gexec, P->stream));
-                PKR_CK(cudaMemcpyAsync(P->hctl, P->ctl, sizeof(RunCtl), cudaMemcpyDeviceToHost,
+                PKR_CK(cudaMemcpyAsync(&P->hctl, P->ctl, sizeof(RunCtl), cudaMemcpyDeviceToHost,
                                        P->stream));
                 PKR_CK(cudaStreamSynchronize(P->stream));
-                const RunCtl c = *P->hctl;
+                const RunCtl c = P->hctl;
                 const int64_t ran = c.stop ? (int64_t)c.done_at + 1 : (int64_t)kGraphSteps;
                 P->launches += ran;
                 done += ran;

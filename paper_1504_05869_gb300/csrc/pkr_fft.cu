@@ -236,32 +236,27 @@ extern "C" int pkr_fixed_point_fft(const pkr_problem* p, const double* rho, doub
 
     const int nxh = nx / 2 + 1;
     const size_t nspec = (size_t)nxh * ny * nz;
-    double* d_r = nullptr;              // source, then Phi
-    cufftDoubleComplex* d_k = nullptr;  // half spectrum (first holds host rho: 16 nspec >= 8 V)
-    double* d_mean = nullptr;
-    double* d_part = nullptr;
-    int* d_flag = nullptr;
-    double2* d_h = nullptr;             // half-angle phase tables of x, y, z
+    // one device block: source, then Phi; half spectrum (first holds host rho:
+    // 16 nspec >= 8 V); half-angle phase tables of x, y, z; mean, flag, partials
     const int red_blocks = 152 * 4;
-    if (cudaMalloc((void**)&d_r, (size_t)V * 8) != cudaSuccess ||
-        cudaMalloc((void**)&d_k, nspec * sizeof(cufftDoubleComplex)) != cudaSuccess ||
-        cudaMalloc((void**)&d_mean, 8) != cudaSuccess ||
-        cudaMalloc((void**)&d_part, red_blocks * 8) != cudaSuccess ||
-        cudaMalloc((void**)&d_flag, sizeof(int)) != cudaSuccess ||
-        cudaMalloc((void**)&d_h, (size_t)(nx + ny + nz) * sizeof(double2)) != cudaSuccess) {
-        cudaFree(d_h);
-        cudaFree(d_r);
-        cudaFree(d_k);
-        cudaFree(d_mean);
-        cudaFree(d_part);
-        cudaFree(d_flag);
+    const size_t rb = ((size_t)V * 8 + 255) / 256 * 256;
+    const size_t kb = (nspec * sizeof(cufftDoubleComplex) + 255) / 256 * 256;
+    const size_t hb = ((size_t)nx + ny + nz) * sizeof(double2);
+    unsigned char* block = nullptr;
+    if (cudaMalloc((void**)&block, rb + kb + hb + 16 + red_blocks * 8) != cudaSuccess) {
         cudaGetLastError();
         return PKR_ENOMEM;
     }
+    double* d_r = reinterpret_cast<double*>(block);
+    cufftDoubleComplex* d_k = reinterpret_cast<cufftDoubleComplex*>(block + rb);
+    double2* d_h = reinterpret_cast<double2*>(block + rb + kb);
+    double* d_mean = reinterpret_cast<double*>(block + rb + kb + hb);
+    int* d_flag = reinterpret_cast<int*>(d_mean + 1);
+    double* d_part = d_mean + 2;
     cufftHandle fwd = 0, inv = 0;
     bool ok = true;
+    double back[2] = {0.0, 0.0};   // mean, then the flag
     int flag = 0;
-    double mean = 0.0;
     const auto t0 = std::chrono::steady_clock::now();
     {
         const double* rd = rho;
@@ -273,22 +268,17 @@ extern "C" int pkr_fixed_point_fft(const pkr_problem* p, const double* rho, doub
         ok = ok && cudaMemsetAsync(d_flag, 0, sizeof(int), s) == cudaSuccess &&
              launch_rho_partials(rd, V, d_part, red_blocks, d_flag, s) == 0 &&
              launch_finalize_mean(d_part, red_blocks, V, d_mean, s) == 0 &&
-             launch_make_source(rd, d_mean, li.cs2 * (tau - 0.5) / eps, V, d_r, PKR_FP64, s) == 0 &&
-             cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-             cudaMemcpyAsync(&mean, d_mean, sizeof(double), cudaMemcpyDeviceToHost, s) ==
-                 cudaSuccess &&
-             cudaStreamSynchronize(s) == cudaSuccess;
-        ok = ok && !flag;   // a non-finite rho stops here, before phi is written
-        if (ok) {
-            int n3[3] = {nz, ny, nx};
-            const int rank = p->dim;
-            int* dims = n3 + (3 - rank);
-            ok = cufftPlanMany(&fwd, rank, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_D2Z, 1) ==
-                     CUFFT_SUCCESS &&
-                 cufftPlanMany(&inv, rank, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_Z2D, 1) ==
-                     CUFFT_SUCCESS &&
-                 cufftSetStream(fwd, s) == CUFFT_SUCCESS && cufftSetStream(inv, s) == CUFFT_SUCCESS;
-        }
+             launch_make_source(rd, d_mean, li.cs2 * (tau - 0.5) / eps, V, d_r, PKR_FP64, s) == 0;
+        // the transforms of a non-finite rho run for nothing: phi is written
+        // only after the flag has been read.  The inverse plan is built while
+        // the GPU works on the forward transform.
+        int n3[3] = {nz, ny, nx};
+        const int rank = p->dim;
+        int* dims = n3 + (3 - rank);
+        ok = ok &&
+             cufftPlanMany(&fwd, rank, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_D2Z, 1) ==
+                 CUFFT_SUCCESS &&
+             cufftSetStream(fwd, s) == CUFFT_SUCCESS;
         ok = ok && cufftExecD2Z(fwd, d_r, d_k) == CUFFT_SUCCESS;
         if (ok) {
             half_phase_kernel<<<(nx + 255) / 256, 256, 0, s>>>(d_h, nx);
@@ -306,7 +296,16 @@ extern "C" int pkr_fixed_point_fft(const pkr_problem* p, const double* rho, doub
             }
             ok = cudaGetLastError() == cudaSuccess;
         }
-        ok = ok && cufftExecZ2D(inv, d_k, d_r) == CUFFT_SUCCESS;
+        ok = ok &&
+             cufftPlanMany(&inv, rank, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_Z2D, 1) ==
+                 CUFFT_SUCCESS &&
+             cufftSetStream(inv, s) == CUFFT_SUCCESS &&
+             cufftExecZ2D(inv, d_k, d_r) == CUFFT_SUCCESS &&
+             cudaMemcpyAsync(back, d_mean, sizeof(back), cudaMemcpyDeviceToHost, s) ==
+                 cudaSuccess &&
+             cudaStreamSynchronize(s) == cudaSuccess;
+        std::memcpy(&flag, back + 1, sizeof(int));
+        ok = ok && !flag;
         ok = ok && cudaMemcpyAsync(phi, d_r, (size_t)V * 8,
                                    host_buffers ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
                                    s) == cudaSuccess &&
@@ -316,17 +315,12 @@ extern "C" int pkr_fixed_point_fft(const pkr_problem* p, const double* rho, doub
         std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     if (fwd) cufftDestroy(fwd);
     if (inv) cufftDestroy(inv);
-    cudaFree(d_r);
-    cudaFree(d_k);
-    cudaFree(d_mean);
-    cudaFree(d_part);
-    cudaFree(d_flag);
-    cudaFree(d_h);
+    cudaFree(block);
     if (flag) return PKR_EINVAL;
     if (!ok) return PKR_ECUDA;
     if (st) {
         std::memset(st, 0, sizeof(*st));
-        st->rho_mean_removed = mean;
+        st->rho_mean_removed = back[0];
         st->tau_lb = tau;
         st->cs2 = li.cs2;
         st->wall_ms = ms;
