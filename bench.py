@@ -515,12 +515,16 @@ def run(args):
         cpu_full = cpu_full_solve(pk, torch)
 
     if stencil:
-        # binary64 FMA bound: Q FMAs per site; peak from the GB300's nominal
-        # FP64 rate (1.25 TFLOP/s = 625 G FMA/s)
-        fma_s = V * Q / (launch_ms * 1e-3) / 1e9
+        # binary64 pipe bound: about 47 (D3Q111) or 13 (D3Q19) operations per
+        # site in the plane form that 3D grids of this size run, else Q; peak
+        # from the GB300's nominal FP64 rate (1.25 TFLOP/s = 625 G operations/s)
+        planes = LATTICE in ("D3Q111", "D3Q19") and V >= 1 << 20
+        ops = {"D3Q111": 47, "D3Q19": 13}[LATTICE] if planes else Q
+        fma_s = V * ops / (launch_ms * 1e-3) / 1e9
         roofline = {"bound": "alu", "achieved": fma_s, "peak": 625.0, "unit": "GFMA/s",
                     "frac": fma_s / 625.0, "traffic": None, "peak_source": "nominal FP64",
-                    "kernel": f"stencil_kernel<{LATTICE}>", "hbm_gbs": achieved,
+                    "kernel": f"stencil_{'planes_' if planes else ''}kernel<{LATTICE}>",
+                    "hbm_gbs": achieved,
                     "algorithmic_bytes_per_launch": V * bytes_site}
     else:
         roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak,

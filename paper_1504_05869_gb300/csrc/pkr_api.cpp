@@ -204,7 +204,7 @@ struct pkr_plan {
     double host[6]; // read back: [0] mean, [1..4] residual, [5] import mean
     void* slab;     // device block of S, Phi (or the stencil's arrays) and the scratch below
     bool stencil;          // omega = 1, binary64: the state is Phi alone (scalar stencil)
-    int planes;            // stencil mode: z chunk of the plane form, 0: one thread per site
+    int form;              // stencil mode: form of a step (StencilForm)
     double* Ps[2];         // stencil mode: Phi ping-pong
     double* St;            // stencil mode: sum_i chi_i S(x - v_i)
     Coefs<double> cchi;    // stencil mode: chi_c in the weight slot (builds St)
@@ -254,7 +254,7 @@ int launch_stencil_step(pkr_plan* P, const double* in, double* out, const double
     const int nx = (int)n[0], ny = (int)n[1], nz = (int)n[2];
     int rc = 0;
 #define PKR_ST(LL) launch_stencil<LL>(in, out, add, c, P->V, nx, ny, nz, P->small, check, \
-                                      P->partials, P->grid, P->planes, P->stream, P->stop_arg)
+                                      P->partials, P->grid, P->form, P->stream, P->stop_arg)
     switch (P->prob.lattice) {
     case PKR_D1Q5: rc = PKR_ST(D1Q5); break;
     case PKR_D1Q9: rc = PKR_ST(D1Q9); break;
@@ -441,6 +441,9 @@ static_assert(sizeof(RunCtl) <= 64, "the counter sits at byte 64");
 // Steps per launch of a resident run: tens of milliseconds at most.
 constexpr int64_t kResidentSteps = 8192;
 
+// Tiles of 32 sites per SM up to which the stencil's resident forms take a grid.
+constexpr int kStencilTiles = 4;
+
 // Form of a resident run of this plan (0: none).  Only where the plan's
 // one-step kernel computes the same values: the per-site stencil, or the
 // library's own choice of sweep geometry.  Tiles: 4 per SM for the stencil,
@@ -449,9 +452,10 @@ int resident_of(pkr_plan* P)
 {
     if (P->resident >= 0) return P->resident;
     P->resident = 0;
-    if (P->prob.precision != PKR_FP64 || P->prob.variant >= 0 || (P->stencil && P->planes > 0))
+    if (P->prob.precision != PKR_FP64 || P->prob.variant >= 0 ||
+        (P->stencil && P->form != kStencilParts4))
         return 0;
-    const int st = P->stencil ? 1 : 0, most = (st ? 4 : 2) * P->nsm;
+    const int st = P->stencil ? 1 : 0, most = (st ? kStencilTiles : 2) * P->nsm;
     switch (P->prob.lattice) {
     case PKR_D1Q5: P->resident = resident_form<D1Q5>(P->V, st, P->nsm, most); break;
     case PKR_D1Q9: P->resident = resident_form<D1Q9>(P->V, st, P->nsm, most); break;
@@ -588,37 +592,42 @@ int capture_steps(pkr_plan* P, double tol, int tol_kind)
     return PKR_OK;
 }
 
-// Form and grid of the scalar stencil.  3D sets on grids that give every SM
-// a plane tile take the plane form, in chunks of z: the chunk length with the
-// least work on the busiest SM, a chunk costing its planes and about four
-// more for the 2 R partial ones around it (256^3: seven chunks of 37 planes,
-// 1.69 ms a step; five of 52, the fewest with four blocks per SM, 1.88 ms).
-// Other grids take one thread per site.
+// Form and grid of the scalar stencil.  3D sets beyond the resident forms take
+// the plane form (tiles of 32 x 16 or 32 x 8 sites, a chunk of z each) or one
+// thread per site, whichever keeps the busiest SM for the shorter time: a
+// chunk of cz planes costs its planes and the partial ones around it.  The
+// costs are measured (GB300, us per plane and tile and per site of an SM, both
+// sets, grids of 216,000 to 16.8 M sites; an SM's only tile runs an eighth
+// slower).  The two are even at 45 x 60 x 80 (56 us a step against 54, or 89 with
+// an unlucky chunk length); 62 x 163 x 53 takes 124 against 87 (32 x 8, cz 8;
+// 148 with cz 7 in 32 x 16, which leaves most SMs one tile and some two).
 void stencil_geometry(pkr_plan* P)
 {
     const int64_t* n = P->prob.n;
-    P->planes = 0;
-    if (P->lat.dim == 3 && !P->small) {
-        const int64_t tiles = ((n[0] + 31) / 32) * ((n[1] + 15) / 16);
-        int64_t best = 0, items = 0;
-        for (int64_t cz = n[2]; cz >= 6 || cz == n[2]; --cz) {
-            const int64_t it = tiles * ((n[2] + cz - 1) / cz);
-            const int64_t cost = ((it + P->nsm - 1) / P->nsm) * (cz + 4);
-            if (it >= P->nsm && (best == 0 || cost < best)) {
-                best = cost;
-                items = it;
-                P->planes = (int)cz;
-            }
-        }
-        if (P->planes > 0) {
-            P->grid = (int)(items < kMaxGridBlocks ? items : kMaxGridBlocks);
-            return;
-        }
-    }
+    P->form = (P->V + 31) / 32 <= (int64_t)kStencilTiles * P->nsm ? kStencilParts4 : kStencilChain;
     const int tb = stencil_block(P->V, P->nsm);
     int64_t g = (P->V + tb - 1) / tb;
     if (g > (int64_t)P->nsm * 8) g = (int64_t)P->nsm * 8;
     P->grid = (int)g;
+    if (P->lat.dim != 3 || P->small || P->form == kStencilParts4) return;
+    const bool wide = P->lat.reach > 1;
+    const double site = wide ? 0.035 : 0.0074, extra = wide ? 4.5 : 2.0;
+    double best = 0.97 * site * (double)P->V / P->nsm;
+    for (int ty = 16; ty >= 8; ty -= 8) {
+        const double plane = wide ? (ty == 16 ? 6.6 : 3.45) : (ty == 16 ? 2.15 : 1.18);
+        const int64_t tiles = ((n[0] + 31) / 32) * ((n[1] + ty - 1) / ty);
+        for (int64_t cz = n[2] < 4096 ? n[2] : 4096; cz >= 5 || cz == n[2]; --cz) {
+            const int64_t items = tiles * ((n[2] + cz - 1) / cz);
+            const int64_t each = (items + P->nsm - 1) / P->nsm;
+            const double cost =
+                (double)each * ((double)cz + extra) * plane * (each == 1 ? 1.12 : 1.0);
+            if (cost < best) {
+                best = cost;
+                P->form = stencil_planes((int)cz, ty);
+                P->grid = (int)(items < kMaxGridBlocks ? items : kMaxGridBlocks);
+            }
+        }
+    }
 }
 
 size_t plan_bytes(const pkr_problem* p, const LatticeInfo& li, int64_t V, int grid_max)

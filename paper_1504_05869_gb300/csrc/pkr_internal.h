@@ -122,6 +122,14 @@ struct RunCtl {
     double last_res;  // last checked residual
 };
 
+// Form of a scalar stencil step (pkr_stencil.cuh): one thread per site, in one
+// chain or in the parts of the resident forms; or, above these, the plane form
+// with a chunk of cz planes and tiles of ty rows (8 or 16).
+enum StencilForm { kStencilChain = 0, kStencilParts4 = -1 };
+constexpr int stencil_planes(int cz, int ty) { return cz * 32 + ty; }
+constexpr int stencil_cz(int form) { return form / 32; }
+constexpr int stencil_ty(int form) { return form % 32; }
+
 // A resident run (pkr_resident.cuh): up to nsteps check steps in one launch.
 struct CoopArgs {
     double* P[3];            // stencil: the two Phi arrays; sweep: three population arrays

@@ -141,7 +141,11 @@ __device__ __forceinline__ void stencil_partials(double d2, double n2, double mx
 }
 
 // One thread per site; the Q neighbour reads hit L1/L2.  Any grid and set.
-template <class L>
+// SPLIT: the parts of the resident forms, four short chains, for grids that
+// those take (they wait on latency).  Else the binary64 pipe is the bound and
+// one chain of Q multiply-adds from St on has the fewest operations (D3Q111:
+// 111 against 115, D3Q19: 19 against 23).
+template <class L, bool SPLIT>
 __global__ void __launch_bounds__(256)
 stencil_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
                const double* __restrict__ St, const Coefs<double> c, int64_t V, int nx, int ny,
@@ -154,14 +158,22 @@ stencil_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
         const int s = (int)s64;
         Neighbours<L> nb;
         nb.locate(s, nx, ny, nz, small);
-        double a[kStencilParts];
-        static_for<0, kStencilParts>([&](auto J) {
-            constexpr int j = decltype(J)::value;
-            a[j] = stencil_part<L, j>(c, [&](auto I) {
-                return __ldg(Pin + nb.template at<decltype(I)::value>());
+        double acc = St ? St[s] : 0.0;
+        if constexpr (SPLIT) {
+            double a[kStencilParts];
+            static_for<0, kStencilParts>([&](auto J) {
+                constexpr int j = decltype(J)::value;
+                a[j] = stencil_part<L, j>(c, [&](auto I) {
+                    return __ldg(Pin + nb.template at<decltype(I)::value>());
+                });
             });
-        });
-        const double acc = ((a[0] + a[1]) + (a[2] + a[3])) + (St ? St[s] : 0.0);
+            acc = ((a[0] + a[1]) + (a[2] + a[3])) + acc;
+        } else {
+            static_for<0, L::Q>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                acc = fma(c.wphi[cls_of<L>(i)], __ldg(Pin + nb.template at<i>()), acc);
+            });
+        }
         Pout[s] = acc;
         if (check) {
             const double d = acc - Pin[s];
@@ -185,9 +197,12 @@ stencil_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
 // binary64 operations per site of D3Q111: 3 (X) + 15 (R) + 19 (T) + 8, about
 // 47 with the X sums of the rows around the tile, against 111 multiply-adds
 // in the per-site form: 256^3 takes 1.69 ms a step (9.9 GLUPS) against 3.56 ms
-// (4.7).  The tile is 32 x 16 sites, 256 threads of two sites:
-// wide enough that those rows cost 3 x 6/16 operations more, small enough
-// that several blocks share an SM and cover each other's barriers.
+// (4.7).  The tile is 32 x 16 sites, 256 threads of two sites: wide enough
+// that those rows cost 3 x 6/16 operations more, small enough that several
+// blocks share an SM and cover each other's barriers; or 32 x 8, one site a
+// thread, a few percent dearer per site and twice as fine, which fills the SMs
+// more evenly on mid-size grids (100^3: 171 us a step against 179 and, one
+// thread per site, 235; 62 x 163 x 53: 87 against 97 and 124).
 // ---------------------------------------------------------------------------
 // weight class of (a, b, c), any order and sign; -1: not in the set
 template <class L>
@@ -206,16 +221,16 @@ __host__ __device__ constexpr bool ring_used(int a, int b)
     return false;
 }
 
-template <class L>
+template <class L, int TY_>
 struct Planes {
     static constexpr int RC = reach_of<L>();
-    static constexpr int TX = 32, TY = 16, NT = 256;
+    static constexpr int TX = 32, TY = TY_, NT = 256, NH = TX * TY / NT;
     static constexpr int PX = TX + 2 * RC, PY = TY + 2 * RC;
     static constexpr int NLD = (PX * PY + NT - 1) / NT;   // values a thread loads per plane
     static constexpr int NXS = (TX * PY + NT - 1) / NT;   // X positions a thread forms
 };
 
-template <class L>
+template <class L, int TY_>
 __global__ void __launch_bounds__(256, 3)
 stencil_planes_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
                       const double* __restrict__ St, const Coefs<double> c, int nx, int ny,
@@ -223,13 +238,13 @@ stencil_planes_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
                       const int* stop)
 {
     if (stop != nullptr && *stop != 0) return;   // the run stopped before this step
-    using PL = Planes<L>;
-    constexpr int RC = PL::RC, TX = PL::TX, TY = PL::TY, NT = PL::NT, PX = PL::PX, PY = PL::PY;
+    using PL = Planes<L, TY_>;
+    constexpr int NH = PL::NH, RC = PL::RC, TX = PL::TX, TY = PL::TY, NT = PL::NT, PX = PL::PX, PY = PL::PY;
     constexpr int W = 2 * RC + 1;
     __shared__ double ph[PY][PX];
     __shared__ double xsum[RC][PY][TX];
     const int tid = threadIdx.x;
-    const int lx = tid & 31, ly = tid >> 5;     // sites (lx, ly) and (lx, ly + 8)
+    const int lx = tid & 31, ly = tid >> 5;     // site (lx, ly), and (lx, ly + 8) of 16 rows
     const int64_t nxy = (int64_t)nx * ny;
     double d2 = 0.0, n2 = 0.0, mx = 0.0, ms = 0.0;
 
@@ -252,9 +267,11 @@ stencil_planes_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
             for (int k = 0; k < PL::NLD; ++k)
                 if (tid + k * NT < PX * PY) next[k] = __ldg(src + off[k]);
         };
-        double acc[2][W];   // open results of planes z - R .. z + R
+        double acc[NH][W];   // open results of planes z - R .. z + R
 #pragma unroll
-        for (int q = 0; q < W; ++q) acc[0][q] = acc[1][q] = 0.0;
+        for (int h = 0; h < NH; ++h)
+#pragma unroll
+            for (int q = 0; q < W; ++q) acc[h][q] = 0.0;
         fetch(z0 - RC);
         for (int z = z0 - RC; z < z1 + RC; ++z) {
             __syncthreads();   // the previous plane's sums have been read
@@ -280,7 +297,7 @@ stencil_planes_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
             for (int q = 0; q <= RC; ++q)
                 need[q] = (z - q >= z0 && z - q < z1) || (z + q >= z0 && z + q < z1);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < NH; ++h) {
                 const int ry = ly + 8 * h + RC, cx = lx + RC;
                 // R_ab, a >= b: the images of (+-a, +-b) and (+-b, +-a)
                 double R[RC + 1][RC + 1];
@@ -320,7 +337,7 @@ stencil_planes_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
             // the result of plane z - R is complete
             const int zo = z - RC;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < NH; ++h) {
                 const int x = x0 + lx, y = y0 + ly + 8 * h;
                 if (zo >= z0 && x < nx && y < ny) {
                     const int64_t s = nxy * zo + (int64_t)y * nx + x;
@@ -349,21 +366,24 @@ stencil_planes_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
 template <class L>
 int launch_stencil(const double* Pin, double* Pout, const double* St, const Coefs<double>& c,
                    int64_t V, int nx, int ny, int nz, int small, int check, double* partials,
-                   int grid, int planes, void* stream, const int* stop)
+                   int grid, int form, void* stream, const int* stop)
 {
     if constexpr (L::DIM == 3) {
-        if (planes > 0) {   // planes: z chunk of a block (stencil_geometry)
-            using PL = Planes<L>;
-            const int tx = (nx + PL::TX - 1) / PL::TX, ty = (ny + PL::TY - 1) / PL::TY;
-            const int items = tx * ty * ((nz + planes - 1) / planes);
-            stencil_planes_kernel<L><<<grid, PL::NT, 0, (cudaStream_t)stream>>>(
-                Pin, Pout, St, c, nx, ny, nz, tx, ty, planes, items, check, partials, stop);
+        if (form > 0) {
+            const int cz = stencil_cz(form), rows = stencil_ty(form);
+            const int tx = (nx + 31) / 32, ty = (ny + rows - 1) / rows;
+            const int items = tx * ty * ((nz + cz - 1) / cz);
+            const auto kern =
+                rows == 16 ? stencil_planes_kernel<L, 16> : stencil_planes_kernel<L, 8>;
+            kern<<<grid, 256, 0, (cudaStream_t)stream>>>(Pin, Pout, St, c, nx, ny, nz, tx, ty,
+                                                         cz, items, check, partials, stop);
             return (int)cudaGetLastError();
         }
     }
     const int block = (int64_t)grid * 64 >= V ? 64 : 256;   // see stencil_block
-    stencil_kernel<L><<<grid, block, 0, (cudaStream_t)stream>>>(Pin, Pout, St, c, V, nx, ny, nz,
-                                                                small, check, partials, stop);
+    const auto kern = form == kStencilParts4 ? stencil_kernel<L, true> : stencil_kernel<L, false>;
+    kern<<<grid, block, 0, (cudaStream_t)stream>>>(Pin, Pout, St, c, V, nx, ny, nz, small, check,
+                                                   partials, stop);
     return (int)cudaGetLastError();
 }
 

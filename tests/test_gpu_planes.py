@@ -54,3 +54,13 @@ def test_plane_stencil_matches_rolls(pk, lattice, order, shape):
     assert float((got - now).norm() / now.norm()) <= FP64_TOL
     want = float((now - old).norm() / now.norm())
     assert st["residual"] == pytest.approx(want, rel=1e-10)
+
+
+# The finer tiles (32 x 8) and the one-thread-per-site form beyond the resident
+# grids: ragged in every axis, whole tiles in one chunk of z, chunks of fewer
+# planes than the stencil spans (32 x 16), few tiles.
+@pytest.mark.parametrize("lattice,order", [("D3Q111", 5), ("D3Q19", 1)])
+@pytest.mark.parametrize("shape", [(53, 163, 62), (47, 152, 160), (5, 640, 640), (29, 30, 31),
+                                   (17, 200, 47)])
+def test_stencil_forms_match_rolls(pk, lattice, order, shape):
+    test_plane_stencil_matches_rolls(pk, lattice, order, shape)
