@@ -611,10 +611,10 @@ void stencil_geometry(pkr_plan* P)
     P->grid = (int)g;
     if (P->lat.dim != 3 || P->small || P->form == kStencilParts4) return;
     const bool wide = P->lat.reach > 1;
-    const double site = wide ? 0.035 : 0.0074, extra = wide ? 4.5 : 2.0;
+    const double site = wide ? 0.035 : 0.0066, extra = wide ? 4.5 : 2.5;
     double best = 0.97 * site * (double)P->V / P->nsm;
     for (int ty = 16; ty >= 8; ty -= 8) {
-        const double plane = wide ? (ty == 16 ? 6.6 : 3.45) : (ty == 16 ? 2.15 : 1.18);
+        const double plane = wide ? (ty == 16 ? 6.6 : 3.45) : (ty == 16 ? 2.15 : 1.24);
         const int64_t tiles = ((n[0] + 31) / 32) * ((n[1] + ty - 1) / ty);
         for (int64_t cz = n[2] < 4096 ? n[2] : 4096; cz >= 5 || cz == n[2]; --cz) {
             const int64_t items = tiles * ((n[2] + cz - 1) / cz);

@@ -65,22 +65,29 @@ struct Neighbours {
     static constexpr int WY = L::DIM >= 2 ? W : 1, WZ = L::DIM >= 3 ? W : 1;
     int xs[W], yo[WY], zo[WZ];
 
+    // (signed divisions and one branch on small: with unsigned ones and a choice
+    // per offset the per-site form took 39.9 us a step for 32.9 on 100 x 90 x 80,
+    // D3Q19, in 48 registers for 42)
     __device__ __forceinline__ void locate(int s, int nx, int ny, int nz, int small)
     {
-        const int r = (int)((unsigned)s / (unsigned)nx);
-        const int x = s - r * nx;
-        const int z = (int)((unsigned)r / (unsigned)ny);
-        const int y = r - z * ny;
+        const int x = s % nx, r = s / nx, y = r % ny, z = r / ny;
         const int nxy = nx * ny;
         yo[0] = y * nx;
         zo[0] = z * nxy;
+        if (small) {
 #pragma unroll
-        for (int d = -RC; d <= RC; ++d) {
-            xs[d + RC] = small ? wrap_any(x - d, nx) : wrap_near(x - d, nx);
-            if constexpr (L::DIM >= 2)
-                yo[d + RC] = (small ? wrap_any(y - d, ny) : wrap_near(y - d, ny)) * nx;
-            if constexpr (L::DIM >= 3)
-                zo[d + RC] = (small ? wrap_any(z - d, nz) : wrap_near(z - d, nz)) * nxy;
+            for (int d = -RC; d <= RC; ++d) {
+                xs[d + RC] = wrap_any(x - d, nx);
+                if constexpr (L::DIM >= 2) yo[d + RC] = wrap_any(y - d, ny) * nx;
+                if constexpr (L::DIM >= 3) zo[d + RC] = wrap_any(z - d, nz) * nxy;
+            }
+        } else {
+#pragma unroll
+            for (int d = -RC; d <= RC; ++d) {
+                xs[d + RC] = wrap_near(x - d, nx);
+                if constexpr (L::DIM >= 2) yo[d + RC] = wrap_near(y - d, ny) * nx;
+                if constexpr (L::DIM >= 3) zo[d + RC] = wrap_near(z - d, nz) * nxy;
+            }
         }
     }
     // Keeps the compiler from forming all Q sums of at() ahead of a loop that
