@@ -598,7 +598,7 @@ int capture_steps(pkr_plan* P, double tol, int tol_kind)
 // chunk of cz planes costs its planes and the partial ones around it.  The
 // costs are measured (GB300, us per plane and tile and per site of an SM, both
 // sets, grids of 216,000 to 16.8 M sites; an SM's only tile runs an eighth
-// slower).  The two are even at 45 x 60 x 80 (56 us a step against 54, or 89 with
+// slower).  The two are even at 45 x 60 x 80 (54 us a step both ways, or 89 with
 // an unlucky chunk length); 62 x 163 x 53 takes 124 against 87 (32 x 8, cz 8;
 // 148 with cz 7 in 32 x 16, which leaves most SMs one tile and some two).
 void stencil_geometry(pkr_plan* P)
