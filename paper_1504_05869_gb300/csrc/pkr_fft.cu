@@ -11,10 +11,11 @@
 // sums are real: 2 Re over one velocity of each pair (the rest velocity once).
 // The denominator is small near k = 0 (it vanishes like |k|^2); since the phi_i
 // sum to one it is written as sum_i phi_i Re[(1 - e_i) / (1 - (1 - w) e_i)]
-// with 1 - cos(theta) = 2 sin^2(theta / 2), so no term cancels.  The phase
-// theta = k.v_i is reduced exactly on the integers (m v mod n) and its half
-// angle built from per-axis tables of exp(-i pi j / n).  The inverse
-// transform's 1 / V goes into T.
+// with 1 - cos(theta) = 2 sin^2(theta / 2), so nothing cancels there; nor does
+// it near theta = pi, where 1 - (1 - w) e_i vanishes as w nears 2 (see
+// transfer_kernel).  The phase theta = k.v_i is reduced exactly on the integers
+// (m v mod n) and its half angle built from per-axis tables of exp(-i pi j / n).
+// The inverse transform's 1 / V goes into T.
 // The transforms are cuFFT's; the transfer function T(k) is this file's kernel.
 #include <cuda_runtime.h>
 #include <cufft.h>
@@ -47,17 +48,24 @@ __global__ void half_phase_kernel(double2* __restrict__ H, int n)
 
 // Multiply the half spectrum S(k) (nx/2 + 1 modes along x) by T(k) * scale.
 //
-// With theta = k.v, o = 1 - cos(theta) = 2 sin^2(theta / 2) and c = 1 - w,
-//     |1 - c e|^2 = w^2 + 2 c o =: m,
-//     Re q = (w - o) / m,   Re[(1 - e) / (1 - c e)] = (1 + c) o / m,
-// so a velocity needs only sin(theta / 2) and one reciprocal, and nothing
-// cancels near k = 0.  The sets are symmetric under the reflection of every
-// axis: T is too, and one thread forms it for the modes (mx, +-my, +-mz); and
-// the sines of a triple's sign images (+-a, +-b, +-c) share their products.
-// Bound by the binary64 pipe: about 16 operations per +-v pair (35 when each
+// With theta = k.v, s = sin(theta / 2), C = cos(theta / 2), c = 1 - w and
+// d = 1 + c = 2 - w,
+//     |1 - c e|^2 = w^2 + 4 c s^2 = d^2 - 4 c C^2 =: m,
+//     Re q = (w - 2 s^2) / m,   Re[(1 - e) / (1 - c e)] = 2 d s^2 / m.
+// Each sum is taken in the form whose terms have one sign: for w <= 1 m from s,
+// and per class W = sum 1 / m and U = sum s^2 / m (sum Re q = w W - 2 U); for
+// w > 1 (OVER) m from C, and U alone: since w^2 W = n + 4 (w - 1) U for n
+// velocities, sum Re q = (n - 2 d U) / w.  With the first form for w > 1, m is
+// the difference of two numbers near 4 where theta nears pi and w nears 2: T
+// of D3Q111, order 1, at tau_lb = 0.5005 would be off by up to 4e-10 of its
+// value, against 2e-14 (binary64 against 60 digits, modes of 24 x 20 x 18).
+// The sets are symmetric under the reflection of every axis: T is too, and one
+// thread forms it for the modes (mx, +-my, +-mz); and the sines and cosines of
+// a triple's sign images (+-a, +-b, +-c) share their products.  Bound by the
+// binary64 pipe: about 16 operations per +-v pair, 18 for w > 1 (35 when each
 // mode and pair multiplied three phases and divided), for a quarter of the
 // half spectrum.  pkr_fixed_point_fft on 200 x 180 x 150, D3Q111: 12.8 ms
-// before, 3.9 ms now, most of it cuFFT and its plans.
+// before, 3.7 ms now, most of it cuFFT and its plans.
 template <class L>
 struct Triples {   // velocities with no negative component
     static constexpr int reach = L::T.reach;
@@ -105,7 +113,7 @@ __device__ __forceinline__ void axis_phases(const double2* __restrict__ H, int m
     }
 }
 
-template <class L>
+template <class L, bool OVER>
 __global__ void __launch_bounds__(128)
 transfer_kernel(cufftDoubleComplex* __restrict__ sk, int nx, int ny, int nz, const FftCoefs c,
                 const double2* __restrict__ Hx, const double2* __restrict__ Hy,
@@ -115,7 +123,8 @@ transfer_kernel(cufftDoubleComplex* __restrict__ sk, int nx, int ny, int nz, con
     const int nxh = nx / 2 + 1, nyh = ny / 2 + 1, nzh = nz / 2 + 1;
     const int64_t total = (int64_t)nxh * nyh * nzh;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const double w = c.omega, cw = 1.0 - w, w2 = w * w, cw4 = 4.0 * cw;
+    const double w = c.omega, cw = 1.0 - w, d = 2.0 - w, d4 = 4.0 * d;
+    const double m0 = OVER ? d * d : w * w, m1 = OVER ? -4.0 * cw : 4.0 * cw;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
         const int mx = (int)(t % nxh);
         const int64_t r = t / nxh;
@@ -125,51 +134,58 @@ transfer_kernel(cufftDoubleComplex* __restrict__ sk, int nx, int ny, int nz, con
         axis_phases<RY>(Hy, my, ny, cy, sy);
         axis_phases<RZ>(Hz, mz, nz, cz, sz);
         double num = 0.0, den = 0.0, U = 0.0, W = 0.0;
-        // one sine: U += s^2 / m, W += 1 / m; two share their reciprocal
-        auto one = [&](double s) {
-            const double q = s * s, inv = 1.0 / fma(cw4, q, w2);
+        int count = 0;   // velocities of the class so far
+        // one half angle (s, C); two share their reciprocal
+        auto one = [&](double s, double C) {
+            const double q = s * s, inv = 1.0 / fma(m1, OVER ? C * C : q, m0);
             U = fma(q, inv, U);
-            W += inv;
+            if constexpr (!OVER) W += inv;
         };
-        auto two = [&](double s, double p) {
+        auto two = [&](double s, double C, double p, double D) {
             const double qs = s * s, qp = p * p;
-            const double ms = fma(cw4, qs, w2), mp = fma(cw4, qp, w2);
+            const double ms = fma(m1, OVER ? C * C : qs, m0);
+            const double mp = fma(m1, OVER ? D * D : qp, m0);
             const double inv = 1.0 / (ms * mp);
             const double is = inv * mp, ip = inv * ms;
             U = fma(qs, is, fma(qp, ip, U));
-            W += is + ip;
+            if constexpr (!OVER) W += is + ip;
         };
         unroll<0, Triples<L>::count()>([&](auto K) {
             constexpr int k = decltype(K)::value;
             constexpr int cl = Triples<L>::cls(k);
-            constexpr int a = Triples<L>::v(k).x, b = Triples<L>::v(k).y, d = Triples<L>::v(k).z;
-            if constexpr (a == 0 && b == 0 && d == 0) {
-                num = c.chi[cl] / w;   // the rest velocity: o = 0, m = w^2
-            } else if constexpr ((a > 0) + (b > 0) + (d > 0) == 1) {
-                one(a > 0 ? sx[a] : b > 0 ? sy[b] : sz[d]);
-            } else if constexpr ((a > 0) + (b > 0) + (d > 0) == 2) {
+            constexpr int a = Triples<L>::v(k).x, b = Triples<L>::v(k).y, e = Triples<L>::v(k).z;
+            constexpr int axes = (a > 0) + (b > 0) + (e > 0);
+            if constexpr (axes == 0) {
+                if constexpr (!OVER) num = c.chi[cl] / w;   // the rest velocity: s = 0, m = w^2
+            } else if constexpr (axes == 1) {
+                one(a > 0 ? sx[a] : b > 0 ? sy[b] : sz[e], a > 0 ? cx[a] : b > 0 ? cy[b] : cz[e]);
+            } else if constexpr (axes == 2) {
                 const double c1 = a > 0 ? cx[a] : cy[b], s1 = a > 0 ? sx[a] : sy[b];
-                const double c2 = d > 0 ? cz[d] : cy[b], s2 = d > 0 ? sz[d] : sy[b];
-                const double p = s1 * c2, q = c1 * s2;
-                two(p + q, p - q);
+                const double c2 = e > 0 ? cz[e] : cy[b], s2 = e > 0 ? sz[e] : sy[b];
+                const double p = s1 * c2, q = c1 * s2, u = c1 * c2, v = s1 * s2;
+                two(p + q, u - v, p - q, u + v);
             } else {
-                // y and z first: angles b + d and b - d, then both with +-a
-                const double p = sy[b] * cz[d], q = cy[b] * sz[d];
-                const double u = cy[b] * cz[d], v = sy[b] * sz[d];
+                // y and z first: angles b + e and b - e, then both with +-a
+                const double p = sy[b] * cz[e], q = cy[b] * sz[e];
+                const double u = cy[b] * cz[e], v = sy[b] * sz[e];
                 const double sp = p + q, sm = p - q, cp = u - v, cm = u + v;
-                const double e = sx[a] * cp, f = cx[a] * sp, g = sx[a] * cm, h = cx[a] * sm;
-                two(e + f, e - f);
-                two(g + h, g - h);
+                const double f1 = sx[a] * cp, f2 = cx[a] * sp, g1 = cx[a] * cp, g2 = sx[a] * sp;
+                two(f1 + f2, g1 - g2, f1 - f2, g1 + g2);
+                const double h1 = sx[a] * cm, h2 = cx[a] * sm, i1 = cx[a] * cm, i2 = sx[a] * sm;
+                two(h1 + h2, i1 - i2, h1 - h2, i1 + i2);
             }
-            // the class is complete: two velocities per sine
+            // the class is complete: 2^axes velocities per triple, two per half angle
+            count += 1 << axes;
             if constexpr (Triples<L>::cls(k + 1) != cl) {
-                num += 2.0 * c.chi[cl] * (w * W - 2.0 * U);
+                if constexpr (OVER) num = fma(c.chi[cl], count - d4 * U, num);   // w num
+                else if constexpr (axes > 0) num += 2.0 * c.chi[cl] * (w * W - 2.0 * U);
                 den += c.phi[cl] * U;
                 U = W = 0.0;
+                count = 0;
             }
         });
         const bool zero = mx == 0 && my == 0 && mz == 0;
-        const double T = zero ? 0.0 : num / (4.0 * (1.0 + cw) * den) * c.scale;
+        const double T = zero ? 0.0 : num / ((OVER ? w * d4 : d4) * den) * c.scale;
         const int ya = my, yb = my == 0 || 2 * my == ny ? my : ny - my;
         const int za = mz, zb = mz == 0 || 2 * mz == nz ? mz : nz - mz;
         auto apply = [&](int y, int z) {
@@ -195,7 +211,8 @@ void launch_transfer(cufftDoubleComplex* sk, int nx, int ny, int nz, const FftCo
     const int64_t total = (int64_t)(nx / 2 + 1) * (ny / 2 + 1) * (nz / 2 + 1);
     int64_t blocks = (total + 127) / 128;
     if (blocks > 152 * 64) blocks = 152 * 64;
-    transfer_kernel<L><<<(int)blocks, 128, 0, s>>>(sk, nx, ny, nz, c, h, h + nx, h + nx + ny);
+    const auto kern = c.omega > 1.0 ? transfer_kernel<L, true> : transfer_kernel<L, false>;
+    kern<<<(int)blocks, 128, 0, s>>>(sk, nx, ny, nz, c, h, h + nx, h + nx + ny);
 }
 
 }  // namespace
