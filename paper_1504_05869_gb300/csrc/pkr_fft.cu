@@ -282,12 +282,15 @@ extern "C" int pkr_fixed_point_fft(const pkr_problem* p, const double* rho, doub
             rd = reinterpret_cast<const double*>(d_k);
         }
         // S = (rho - <rho>) c_s^2 (tau_lb - 1/2) / eps, into d_r
-        ok = ok && cudaMemsetAsync(d_flag, 0, sizeof(int), s) == cudaSuccess &&
-             launch_rho_partials(rd, V, d_part, red_blocks, d_flag, s) == 0 &&
-             launch_finalize_mean(d_part, red_blocks, V, d_mean, s) == 0 &&
-             launch_make_source(rd, d_mean, li.cs2 * (tau - 0.5) / eps, V, d_r, PKR_FP64, s) == 0;
-        // the transforms of a non-finite rho run for nothing: phi is written
-        // only after the flag has been read.  The inverse plan is built while
+        const bool prepared =
+            ok && cudaMemsetAsync(d_flag, 0, sizeof(int), s) == cudaSuccess &&
+            launch_rho_partials(rd, V, d_part, red_blocks, d_flag, s) == 0 &&
+            launch_finalize_mean(d_part, red_blocks, V, d_mean, s) == 0 &&
+            launch_make_source(rd, d_mean, li.cs2 * (tau - 0.5) / eps, V, d_r, PKR_FP64, s) == 0;
+        ok = prepared;
+        // the transforms of a non-finite rho run for nothing, or fail for want
+        // of work space: phi is written only after the flag has been read, and
+        // the flag decides the status first.  The inverse plan is built while
         // the GPU works on the forward transform.
         int n3[3] = {nz, ny, nx};
         const int rank = p->dim;
@@ -317,12 +320,13 @@ extern "C" int pkr_fixed_point_fft(const pkr_problem* p, const double* rho, doub
              cufftPlanMany(&inv, rank, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_Z2D, 1) ==
                  CUFFT_SUCCESS &&
              cufftSetStream(inv, s) == CUFFT_SUCCESS &&
-             cufftExecZ2D(inv, d_k, d_r) == CUFFT_SUCCESS &&
-             cudaMemcpyAsync(back, d_mean, sizeof(back), cudaMemcpyDeviceToHost, s) ==
-                 cudaSuccess &&
-             cudaStreamSynchronize(s) == cudaSuccess;
+             cufftExecZ2D(inv, d_k, d_r) == CUFFT_SUCCESS;
+        const bool read = prepared &&
+                          cudaMemcpyAsync(back, d_mean, sizeof(back), cudaMemcpyDeviceToHost, s) ==
+                              cudaSuccess &&
+                          cudaStreamSynchronize(s) == cudaSuccess;
         std::memcpy(&flag, back + 1, sizeof(int));
-        ok = ok && !flag;
+        ok = ok && read && !flag;
         ok = ok && cudaMemcpyAsync(phi, d_r, (size_t)V * 8,
                                    host_buffers ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
                                    s) == cudaSuccess &&
@@ -333,6 +337,7 @@ extern "C" int pkr_fixed_point_fft(const pkr_problem* p, const double* rho, doub
     if (fwd) cufftDestroy(fwd);
     if (inv) cufftDestroy(inv);
     cudaFree(block);
+    if (!ok) cudaGetLastError();   // an allocation cuFFT was refused is not the next call's error
     if (flag) return PKR_EINVAL;
     if (!ok) return PKR_ECUDA;
     if (st) {
