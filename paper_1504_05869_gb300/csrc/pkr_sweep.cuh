@@ -519,51 +519,58 @@ __device__ __forceinline__ void group_compute(const TileGrid<T>& tg,
 
     // relax and store this group's velocities, one symmetry class at a
     // time (velocities of a class are contiguous and share phi_c, chi_c)
-    static_for<0, NC>([&](auto CI) {
+    auto relax = [&](auto CI) {
         constexpr int cl = decltype(CI)::value;
         constexpr int cb = cls_begin<L>(cl), ce = cls_begin<L>(cl + 1);
         constexpr int i0 = cb > lo ? cb : lo;
         constexpr int i1 = ce < hi ? ce : hi;
-        if (valid) {
-            if constexpr (i0 < i1 && std::is_same<T, long long>::value) {
-                const double e = fma(c.wphi[cl], Phi, c.chi[cl] * Sx);
-                const long long ei = __double2ll_rn(e * pow2(tg.fw));
-                // the written array's scale is 2^-k that of the read one (k >= 0,
-                // the rescale only lowers it): fold 2^-k into the coefficient
-                const int k = tg.fr - tg.fw;
-                const long long cw = k == 0 ? tg.cfx : ((tg.cfx >> (k - 1)) + 1) >> 1;
-                T* dst = B + ((int64_t)i0 * V + s);
+        if constexpr (i0 < i1 && std::is_same<T, long long>::value) {
+            const double e = fma(c.wphi[cl], Phi, c.chi[cl] * Sx);
+            const long long ei = __double2ll_rn(e * pow2(tg.fw));
+            // the written array's scale is 2^-k that of the read one (k >= 0,
+            // the rescale only lowers it): fold 2^-k into the coefficient
+            const int k = tg.fr - tg.fw;
+            const long long cw = k == 0 ? tg.cfx : ((tg.cfx >> (k - 1)) + 1) >> 1;
+            T* dst = B + ((int64_t)i0 * V + s);
 #pragma unroll 2
-                for (int i = i0; i < i1; ++i) {
-                    const long long p = fx_mul(lds_s64(sbase + (i - lo) * VS), cw) + ei;
-                    fxm |= (unsigned long long)(p ^ (p >> 63));
-                    store_stream(dst, (T)p);
-                    dst += V;
-                }
-            } else if constexpr (i0 < i1) {
-                const R e = fma(c.wphi[cl], Phi, c.chi[cl] * Sx);
-                T* dst = B + ((int64_t)i0 * V + s);
-                int i = i0;
-                for (; i + 3 < i1; i += 4) {
-                    const R g0 = lds_val<T>(sbase + (i + 0 - lo) * VS);
-                    const R g1 = lds_val<T>(sbase + (i + 1 - lo) * VS);
-                    const R g2 = lds_val<T>(sbase + (i + 2 - lo) * VS);
-                    const R g3 = lds_val<T>(sbase + (i + 3 - lo) * VS);
-                    store_stream(dst, (T)fma(c.om1, g0, e));
-                    store_stream(dst + V, (T)fma(c.om1, g1, e));
-                    store_stream(dst + 2 * V, (T)fma(c.om1, g2, e));
-                    store_stream(dst + 3 * V, (T)fma(c.om1, g3, e));
-                    dst += 4 * V;
-                }
-                for (; i < i1; ++i) {
-                    const R gi = lds_val<T>(sbase + (i - lo) * VS);
-                    store_stream(dst, (T)fma(c.om1, gi, e));
-                    dst += V;
-                }
+            for (int i = i0; i < i1; ++i) {
+                const long long p = fx_mul(lds_s64(sbase + (i - lo) * VS), cw) + ei;
+                fxm |= (unsigned long long)(p ^ (p >> 63));
+                store_stream(dst, (T)p);
+                dst += V;
+            }
+        } else if constexpr (i0 < i1) {
+            const R e = fma(c.wphi[cl], Phi, c.chi[cl] * Sx);
+            T* dst = B + ((int64_t)i0 * V + s);
+            int i = i0;
+            for (; i + 3 < i1; i += 4) {
+                const R g0 = lds_val<T>(sbase + (i + 0 - lo) * VS);
+                const R g1 = lds_val<T>(sbase + (i + 1 - lo) * VS);
+                const R g2 = lds_val<T>(sbase + (i + 2 - lo) * VS);
+                const R g3 = lds_val<T>(sbase + (i + 3 - lo) * VS);
+                store_stream(dst, (T)fma(c.om1, g0, e));
+                store_stream(dst + V, (T)fma(c.om1, g1, e));
+                store_stream(dst + 2 * V, (T)fma(c.om1, g2, e));
+                store_stream(dst + 3 * V, (T)fma(c.om1, g3, e));
+                dst += 4 * V;
+            }
+            for (; i < i1; ++i) {
+                const R gi = lds_val<T>(sbase + (i - lo) * VS);
+                store_stream(dst, (T)fma(c.om1, gi, e));
+                dst += V;
             }
         }
-        if constexpr (i0 < i1) after_class(CI);
-    });
+    };
+    if constexpr (std::is_same<Hook, NoHook>::value) {
+        if (valid) static_for<0, NC>(relax);
+    } else {
+        static_for<0, NC>([&](auto CI) {
+            constexpr int cl = decltype(CI)::value;
+            if (valid) relax(CI);
+            // classes the group holds velocities of
+            if constexpr (cls_begin<L>(cl) < hi && cls_begin<L>(cl + 1) > lo) after_class(CI);
+        });
+    }
     // density output and residual contributions (one group per tile)
     if (g == 0 && mode != kPlain && valid) {
         const double ph = (double)Phi;
@@ -634,21 +641,35 @@ __host__ __device__ constexpr int tail_begin(int lo, int hi)
     return b > lo ? b : lo;
 }
 
-// (small sets: D3Q19 at 256^3 17.9 GLUPS with early refill, 18.1 without)
-template <class L, typename T>
+// Where a tile's copies may start while the one before is relaxed (EARLY
+// below): binary64 of the large sets.  GLUPS on 173 x 141 x 100, D3Q111, 2
+// groups x 2 tiles, with and without: binary64 2.67 / 2.37, fixed point 2.88 /
+// 2.95, binary32 5.15 / 5.81; D3Q19 in binary64 at 256^3 17.9 / 18.1.  D2Q169's
+// geometries of few or unpaired warps lose by it (500 x 513, 1 x 2 299 us
+// a step with and 294 without, 3 x 1 219 / 206, 4 x 1 243 / 212; 2 x 2 190 / 209).
+template <class L, typename T, int G, int TILES>
 struct EarlyRefill {
-    static constexpr bool value = L::Q > 64 && std::is_same<T, double>::value;
+    static constexpr bool value = L::Q > 64 && std::is_same<T, double>::value &&
+                                  (L::Q <= 111 || G == 2 || (G == 3 && TILES == 2));
 };
-// One tile of velocity group g.  In binary64 its copies are in flight already,
-// and class by class as it is relaxed the copies of the warp's next tile
+// And when it pays: rounds of tiles per resident warp group.  A block's first
+// tile overlaps nothing, and a grid of one tile each only runs the longer code:
+// time of a step with refill to that without, 2 groups x 2 tiles, by rounds:
+// D3Q111 1.04 (0.9), 1.02 (1.35), 0.99 (1.6), 0.95 (2.2), 0.88 (3.3), 0.87 (14);
+// D2Q81 0.98 (1.3), 0.92 (1.9), 0.86 (3.5); D2Q169, a third fewer warps per SM,
+// 1.09 (1.2), 1.04 (1.5), 1.02 (2.1), 1.01 (3.2), 0.95 (4.6), 0.89 (51).
+template <class L>
+bool early_refill_pays(int64_t ntiles, int64_t slots)
+{
+    return 2 * ntiles >= (L::Q > 111 ? 8 : 3) * slots;
+}
+// One tile of velocity group g.  EARLY: its copies are in flight already, and
+// class by class as it is relaxed the copies of the warp's next tile
 // (`refill(I)` copies velocity I of it) are started, so the pull of a tile
 // overlaps the computation of the one before; each class is a copy group of
 // its own, so a tile starts once every class but its last (refilled last) has
-// landed, as in the x-pairs sweep.  The other storages copy a tile at its
-// start.  GLUPS on 173 x 141 x
-// 100, D3Q111, 2 groups x 2 tiles, early refill against copies at the start:
-// binary64 2.64 / 2.41, fixed point 2.88 / 2.91, binary32 5.15 / 5.56.
-template <class L, typename T, int G, int g, class Refill>
+// landed, as in the x-pairs sweep.  Else refill copies this tile.
+template <class L, typename T, int G, int g, bool EARLY, class Refill>
 __device__ __forceinline__ void tile_compute(const TileGrid<T>& tg,
                                              const Coefs<typename AccType<T>::type>& c, int mode,
                                              bool valid, int s, typename AccType<T>::type Sx,
@@ -661,7 +682,7 @@ __device__ __forceinline__ void tile_compute(const TileGrid<T>& tg,
     constexpr int lo = g * L::Q / G, hi = (g + 1) * L::Q / G;
     constexpr int VS = 32 * (int)sizeof(T);
     constexpr int tb = tail_begin<L>(lo, hi);
-    if constexpr (EarlyRefill<L, T>::value) {
+    if constexpr (EARLY) {
         cp_async_wait_all_but_last();
         group_compute<L, T, G, g, VS, tb - lo>(
             tg, c, mode, valid, s, Sx, lane, sbase, bar, xacc, xexp, d2, n2, mx, ms, fxm,
@@ -688,15 +709,13 @@ __device__ __forceinline__ void tile_first(const Refill& refill)
 {
     constexpr int lo = g * L::Q / G, hi = (g + 1) * L::Q / G;
     constexpr int tb = tail_begin<L>(lo, hi);
-    if constexpr (EarlyRefill<L, T>::value) {
-        static_for<lo, tb>(refill);
-        cp_async_commit();
-        static_for<tb, hi>(refill);
-        cp_async_commit();
-    }
+    static_for<lo, tb>(refill);
+    cp_async_commit();
+    static_for<tb, hi>(refill);
+    cp_async_commit();
 }
 
-template <class L, typename T, int G_, int TILES_>
+template <class L, typename T, int G_, int TILES_, bool EARLY>
 __global__ void __launch_bounds__(G_ * TILES_ * 32)
 sweep_staged_kernel(const SweepArgs a, const Coefs<typename AccType<T>::type> c)
 {
@@ -728,43 +747,56 @@ sweep_staged_kernel(const SweepArgs a, const Coefs<typename AccType<T>::type> c)
     unsigned long long fxm = 0ull;
     const int nt = gridDim.x * TILES;
     int par = 0;
-    static_for<0, G>([&](auto GI) {
+    using R = typename AccType<T>::type;
+    TilePull<L, T> next;
+    auto locate = [&](int tile) {
+        next.locate(tile, tg.V, tg.nx, tg.ny, tg.nz, tg.small, a.zero_in != 0, lane);
+    };
+    // one tile of group g; its copies, or those of the next tile, by refill
+    auto step = [&](auto GI, int tile, const auto& refill) {
         constexpr int g = decltype(GI)::value;
-        if (grp != g) return;
-        using R = typename AccType<T>::type;
-        TilePull<L, T> next;
-        auto refill = [&](auto I) {
+        const int64_t s64 = (int64_t)tile * 32 + lane;
+        const bool valid = s64 < tg.V;
+        const int s = valid ? (int)s64 : 0;
+        // the source offset (mass correction) is used by binary32 storage only
+        R Sx = R(0);
+        if (valid) {
+            if constexpr (std::is_same<T, float>::value) Sx = (R)((double)tg.S[s] + tg.soff);
+            else Sx = (R)tg.S[s];
+        }
+        const bool more = EARLY && tile + nt < a.ntiles;
+        if (more) locate(tile + nt);
+        tile_compute<L, T, G, g, EARLY>(tg, c, a.mode, valid, s, Sx, lane, sbase, 1 + sub,
+                                        xacc[par][sub], xexp[sub], rd2, rn2, rmx, rms, fxm, more,
+                                        refill);
+    };
+    auto refill_of = [&](auto GI) {
+        return [&](auto I) {
             constexpr int i = decltype(I)::value;
-            next.template pull<i>(tg.A, tg.V, sbase + (uint32_t)((i - ST::lo(g)) * 32 * sizeof(T)));
+            constexpr int lo = decltype(GI)::value * L::Q / G;
+            next.template pull<i>(tg.A, tg.V, sbase + (uint32_t)((i - lo) * 32 * sizeof(T)));
         };
-        int tile = blockIdx.x * TILES + sub;
-        if (EarlyRefill<L, T>::value && tile < a.ntiles) {
-            next.locate(tile, tg.V, tg.nx, tg.ny, tg.nz, tg.small, a.zero_in != 0, lane);
-            tile_first<L, T, G, g>(refill);
-        }
+    };
+    int tile = blockIdx.x * TILES + sub;
+    if constexpr (EARLY) {
+        // a group's copies run ahead into its own next tile: a loop for each
+        static_for<0, G>([&](auto GI) {
+            if (grp != decltype(GI)::value) return;
+            const auto refill = refill_of(GI);
+            if (tile < a.ntiles) {
+                locate(tile);
+                tile_first<L, T, G, decltype(GI)::value>(refill);
+            }
+            for (; tile < a.ntiles; tile += nt, par ^= 1) step(GI, tile, refill);
+        });
+    } else {
         for (; tile < a.ntiles; tile += nt, par ^= 1) {
-            const int64_t s64 = (int64_t)tile * 32 + lane;
-            const bool valid = s64 < tg.V;
-            // the source offset (mass correction) is used by binary32 storage only
-            R Sx = R(0);
-            if (valid) {
-                if constexpr (std::is_same<T, float>::value)
-                    Sx = (R)((double)tg.S[s64] + tg.soff);
-                else Sx = (R)tg.S[s64];
-            }
-            const bool more = tile + nt < a.ntiles;
-            if constexpr (EarlyRefill<L, T>::value) {
-                if (more)
-                    next.locate(tile + nt, tg.V, tg.nx, tg.ny, tg.nz, tg.small, a.zero_in != 0,
-                                lane);
-            } else {
-                next.locate(tile, tg.V, tg.nx, tg.ny, tg.nz, tg.small, a.zero_in != 0, lane);
-            }
-            tile_compute<L, T, G, g>(tg, c, a.mode, valid, (int)s64, Sx, lane, sbase, 1 + sub,
-                                     xacc[par][sub], xexp[sub], rd2, rn2, rmx, rms, fxm, more,
-                                     refill);
+            locate(tile);
+            static_for<0, G>([&](auto GI) {
+                if (grp == decltype(GI)::value) step(GI, tile, refill_of(GI));
+            });
         }
-    });
+    }
     if constexpr (std::is_same<T, long long>::value) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -897,29 +929,11 @@ sweep_batch_kernel(BatchState* st, int k, int phase)
             }
         }
     };
-    static_for<0, G>([&](auto GI) {
-        constexpr int g = decltype(GI)::value;
-        if (grp != g) return;
+    // this warp's tiles; groups(f) calls f with the warp's velocity group
+    auto loop = [&](const auto& groups) {
         int tile = blockIdx.x * TILES + sub;
         if (tile >= ntiles) return;
         int gi = grid_of(tile);
-        TilePull<L, T> next;
-        const T* A = nullptr;
-        int64_t V = 0;
-        // tile t of grid gi, whose copies come next
-        auto locate = [&](int t) {
-            const BatchGrid<R>& gd = grids[gi];
-            const long long age = step - gd.join;
-            A = static_cast<const T*>(gd.pop[age & 1]);
-            V = gd.V;
-            next.locate(t - gd.tile_begin, V, gd.nx, gd.ny, gd.nz, gd.small, age == 0, lane);
-        };
-        auto refill = [&](auto I) {
-            constexpr int i = decltype(I)::value;
-            next.template pull<i>(A, V, sbase + (uint32_t)((i - ST::lo(g)) * 32 * sizeof(T)));
-        };
-        if constexpr (EarlyRefill<L, T>::value) locate(tile);
-        tile_first<L, T, G, g>(refill);
         for (; tile < ntiles; tile += nt, par ^= 1) {
             const BatchGrid<R>& gd = grids[gi];
             const long long age = step - gd.join;
@@ -933,21 +947,44 @@ sweep_batch_kernel(BatchState* st, int k, int phase)
                     Sx = (R)((double)tg.S[s64] + tg.soff);
                 else Sx = (R)tg.S[s64];
             }
-            const bool more = tile + nt < ntiles;
-            if constexpr (!EarlyRefill<L, T>::value) locate(tile);
+            TilePull<L, T> here;
+            here.locate(tile - gd.tile_begin, tg.V, tg.nx, tg.ny, tg.nz, tg.small, age == 0, lane);
             // the next tile's grid is this one or a later one
-            if (more)
+            if (tile + nt < ntiles)
                 while (gi + 1 < ngrids && grids[gi + 1].tile_begin <= tile + nt) ++gi;
-            if constexpr (EarlyRefill<L, T>::value) {
-                if (more) locate(tile + nt);
-            }
             double d2 = 0.0, n2 = 0.0, mx = 0.0, ms = 0.0;
             unsigned long long fxm = 0ull;
-            tile_compute<L, T, G, g>(tg, gd.c, mode, valid, (int)s64, Sx, lane, sbase, 1 + sub,
-                                     xacc[par][sub], xexp[sub], d2, n2, mx, ms, fxm, more, refill);
+            groups([&](auto GI) {
+                constexpr int g = decltype(GI)::value;
+                auto pull = [&](auto I) {
+                    constexpr int i = decltype(I)::value;
+                    here.template pull<i>(tg.A, tg.V,
+                                          sbase + (uint32_t)((i - ST::lo(g)) * 32 * sizeof(T)));
+                };
+                tile_compute<L, T, G, g, false>(tg, gd.c, mode, valid, (int)s64, Sx, lane, sbase,
+                                                1 + sub, xacc[par][sub], xexp[sub], d2, n2, mx, ms,
+                                                fxm, false, pull);
+            });
             finish(gd, tile, mode, d2, n2, mx, ms, fxm);
         }
-    });
+    };
+    // One loop for all groups in binary64, one for each in the other storages,
+    // as measured (us per window of 32 steps, one loop / each its own: D3Q111,
+    // 16 grids of 32 x 33 x 34, 2 groups x 2 tiles, binary64 9630 / 9800;
+    // binary32 and fixed point up to 5 % the other way).  No copies ahead of a
+    // tile (EarlyRefill) here: with them the same batch took 10140 us, 32 grids
+    // of 100 x 120 of D2Q169 13560 against 11900.
+    if constexpr (std::is_same<T, double>::value) {
+        loop([&](const auto& f) {
+            static_for<0, G>([&](auto GI) {
+                if (grp == decltype(GI)::value) f(GI);
+            });
+        });
+    } else {
+        static_for<0, G>([&](auto GI) {
+            if (grp == decltype(GI)::value) loop([&](const auto& f) { f(GI); });
+        });
+    }
 }
 
 template <class L, typename T, int K>
@@ -1497,8 +1534,12 @@ int launch_variant(const SweepArgs& a, const void* coefs, int grid, void* stream
     using R = typename AccType<T>::type;
     constexpr Geo geo = Variants<L>::at(K);
     using ST = Staged<L, T, geo.G, geo.TILES>;
-    sweep_staged_kernel<L, T, geo.G, geo.TILES><<<grid, ST::WARPS * 32, ST::smem_bytes(),
-                                                  (cudaStream_t)stream>>>(
+    auto kern = sweep_staged_kernel<L, T, geo.G, geo.TILES, false>;
+    if constexpr (EarlyRefill<L, T, geo.G, geo.TILES>::value) {
+        if (early_refill_pays<L>(a.ntiles, (int64_t)grid * geo.TILES))
+            kern = sweep_staged_kernel<L, T, geo.G, geo.TILES, true>;
+    }
+    kern<<<grid, ST::WARPS * 32, ST::smem_bytes(), (cudaStream_t)stream>>>(
         a, *static_cast<const Coefs<R>*>(coefs));
     return (int)cudaGetLastError();
 }
@@ -1508,12 +1549,21 @@ int occupancy_variant(int* blocks, int* tiles_per_block)
 {
     constexpr Geo geo = Variants<L>::at(K);
     using ST = Staged<L, T, geo.G, geo.TILES>;
-    auto kern = sweep_staged_kernel<L, T, geo.G, geo.TILES>;
-    cudaError_t e = set_sweep_smem(kern, ST::smem_bytes());
-    if (e != cudaSuccess) return (int)e;
-    *tiles_per_block = geo.TILES;
-    return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kern, ST::WARPS * 32,
+    auto residency = [&](auto kern) {
+        int b = 0;
+        cudaError_t e = set_sweep_smem(kern, ST::smem_bytes());
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, ST::WARPS * 32,
                                                               ST::smem_bytes());
+        if (b < *blocks || *blocks == 0) *blocks = b;
+        return e;
+    };
+    *tiles_per_block = geo.TILES;
+    *blocks = 0;
+    cudaError_t e = residency(sweep_staged_kernel<L, T, geo.G, geo.TILES, false>);
+    if constexpr (EarlyRefill<L, T, geo.G, geo.TILES>::value)
+        if (e == cudaSuccess) e = residency(sweep_staged_kernel<L, T, geo.G, geo.TILES, true>);
+    return (int)e;
 }
 
 // Run-time dispatch over the compiled variants of (L, T): the staged
