@@ -112,19 +112,27 @@ int variant_count(int lattice)
 // {(1,2),(1,4)} (D3Q19: the two within 0.2 %).  Large sets whose x rows are
 // whole 64-site pairs take the early-refill x-pairs sweep once the grid
 // gives every block a few pairs (GLUPS, early refill against (2,2): D3Q111
-// at 256^3 3.09 / 2.84 in 64-bit fixed point, 2.61 / 2.50 in binary64, 5.54
-// / 5.38 in binary32; D2Q81 at 2048^2 3.85 / 3.69 and 3.60 / 3.35; D2Q169 at
-// 2048^2 1.44 / 1.33 in binary64 but 1.35 / 1.48 in fixed point, where two
-// blocks of 103 KB per SM leave 28 KB of L1).  Other grids take 2 velocity
-// groups x 2 tiles, or, with few tiles per SM, 4 groups x 1 tile (more warps
-// share each tile, so each step's chain is shorter).  All geometries give
-// the same binary64 result.
+// at 256^3 3.09 / 2.84 in 64-bit fixed point, 2.61 / 2.50 in binary64;
+// D2Q81 at 2048^2 3.85 / 3.69 and 3.60 / 3.35; D2Q169 at 2048^2 1.44 / 1.33 in
+// binary64 but 1.35 / 1.48 in fixed point, where two blocks of 103 KB per SM
+// leave 28 KB of L1): 8 pairs per SM, an SM holding at most 3.
+//   binary32 (two sites per lane) holds 6 pairs per SM and fetches a pair ahead
+// for each: from 22 pairs per SM on, and not D2Q169, of which it holds 3.  Time
+// of a step to that of (2,2), by pairs per SM: D3Q111 1.61 (8), 1.22 (13), 1.03
+// (16), 0.98 (18), 1.05 (20), 0.97 (24), 1.03 (30), 0.99 (36), 0.96 (46), 0.93
+// (65), 0.92 (119); D2Q81 1.62 (8), 1.08 (18), 1.11 (20), 0.98 (24), 1.05 (26),
+// 1.00 (30 to 46), 0.96 (66), 0.92 (431); D2Q169 1.23 (8), 1.09 (24), 1.06 (431).
+//   Other grids take 2 velocity groups x 2 tiles, or, with few tiles per SM,
+// 4 groups x 1 tile (more warps share each tile, so each step's chain is
+// shorter).  All geometries give the same binary64 and fixed-point result, and
+// (2,2) and the x-pairs ones the same binary32 result.
 int default_variant(int lattice, int precision, int64_t V, int nsm, bool xpairs)
 {
     if (variant_count(lattice) <= 2) return 0;
     const int pv = pair_variant(lattice);
-    if (xpairs && pv >= 0 && V / 64 >= (int64_t)8 * nsm &&
-        !(lattice == PKR_D2Q169 && precision == PKR_FX64))
+    const bool f32 = precision == PKR_FP32;
+    if (xpairs && pv >= 0 && V / 64 >= (int64_t)(f32 ? 22 : 8) * nsm &&
+        !(lattice == PKR_D2Q169 && (f32 || precision == PKR_FX64)))
         return pv + 1;
     return (V + 31) / 32 <= (int64_t)4 * nsm ? 5 : 2;
 }
