@@ -274,6 +274,23 @@ int pkr_plan_phi(pkr_plan *plan, double *phi, int phi_on_host);
 /* Steps t completed so far (Phi^t is the latest density). */
 int64_t pkr_plan_steps(const pkr_plan *plan);
 
+/* What a step of the plan launches, as the plan's rules chose it for its grid
+ * (for tests, benchmarks and logs).  form[0]: pkr_step_kind; form[1], form[2]:
+ * its parameters; form[3]: thread blocks of the launch; form[4]: the form of
+ * per-step-checked binary64 runs of 64 steps and more (pkr_plan_run): 0
+ * captured graphs, 1 scalar stencil in one block, 2 scalar stencil in a
+ * cooperative launch, 3 population sweep in a cooperative launch.  Errors:
+ * PKR_EINVAL. */
+typedef enum pkr_step_kind {
+    PKR_STEP_SWEEP = 0,     /* population sweep; form[1]: variant */
+    PKR_STEP_SWEEP16 = 1,   /* binary16 population sweep; form[1]: sites per lane, form[2]: 1
+                               if a tile's copies start while the one before is relaxed */
+    PKR_STEP_STENCIL = 2,   /* scalar stencil, a thread per site; form[1]: partial sums */
+    PKR_STEP_PLANES = 3     /* scalar stencil by planes; form[1]: planes per chunk of z,
+                               form[2]: rows of a tile */
+} pkr_step_kind;
+int pkr_plan_step_form(pkr_plan *plan, int32_t form[5]);
+
 /* Raw access for tests: device pointer of the current population array
  * (Q*V elements of the storage type, plane i at offset i*V) and of Phi. */
 void *pkr_plan_populations(pkr_plan *plan);

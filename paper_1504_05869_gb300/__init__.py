@@ -150,6 +150,13 @@ class Plan:
     def steps(self) -> int:
         return int(_pkr.pkr_plan_steps(self._h))
 
+    def step_form(self) -> tuple:
+        """pkr_plan_step_form: (kind, parameter, parameter, blocks, form of
+        per-step-checked runs)."""
+        form = (ctypes.c_int32 * 5)()
+        check(_pkr.pkr_plan_step_form(self._h, form), "pkr_plan_step_form")
+        return tuple(form)
+
     def populations_ptr(self) -> int:
         return int(_pkr.pkr_plan_populations(self._h) or 0)
 

@@ -24,6 +24,8 @@ LATTICE_DIM = {"D1Q5": 1, "D1Q9": 1, "D1Q13": 1, "D2Q25": 2, "D2Q81": 2, "D2Q169
 PKR_FP64, PKR_FP32, PKR_MIXED, PKR_FP16, PKR_MIXED16, PKR_FX64 = 0, 1, 2, 3, 4, 5
 PKR_MIXED_FX64 = 6
 PKR_TOL_MAX_ABS_DPHI, PKR_TOL_REL_L2_DPHI = 0, 1
+# pkr_step_kind
+PKR_STEP_SWEEP, PKR_STEP_SWEEP16, PKR_STEP_STENCIL, PKR_STEP_PLANES = 0, 1, 2, 3
 
 # Every symbol include/pkr.h declares (checked by the tests).
 EXPORTS = [
@@ -34,7 +36,7 @@ EXPORTS = [
     "pkr_batch_variant_count",
     "pkr_plan_autotune", "pkr_ctx_create", "pkr_submit", "pkr_poll", "pkr_ctx_run",
     "pkr_ctx_wait", "pkr_ctx_info", "pkr_ctx_destroy", "pkr_plan_import",
-    "pkr_fixed_point_fft", "pkr_ctx_release", "pkr_pull_copy_ceiling",
+    "pkr_fixed_point_fft", "pkr_ctx_release", "pkr_pull_copy_ceiling", "pkr_plan_step_form",
 ]
 
 
@@ -88,6 +90,7 @@ _SIGS = {
     "pkr_plan_sweeps": (ctypes.c_int, [_P, ctypes.c_int64]),
     "pkr_plan_phi": (ctypes.c_int, [_P, _P, ctypes.c_int]),
     "pkr_plan_steps": (ctypes.c_int64, [_P]),
+    "pkr_plan_step_form": (ctypes.c_int, [_P, _I32]),
     "pkr_plan_populations": (_P, [_P]),
     "pkr_solve": (ctypes.c_int, [ctypes.POINTER(pkr_problem), _P, _P, ctypes.c_int,
                                  ctypes.POINTER(pkr_stats), _P]),
@@ -163,6 +166,7 @@ pkr_plan_run = _fn("pkr_plan_run")
 pkr_plan_sweeps = _fn("pkr_plan_sweeps")
 pkr_plan_phi = _fn("pkr_plan_phi")
 pkr_plan_steps = _fn("pkr_plan_steps")
+pkr_plan_step_form = _fn("pkr_plan_step_form")
 pkr_plan_populations = _fn("pkr_plan_populations")
 pkr_solve = _fn("pkr_solve")
 pkr_residual_noalloc = _fn("pkr_residual_noalloc")

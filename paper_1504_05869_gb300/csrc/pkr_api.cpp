@@ -1290,6 +1290,29 @@ int pkr_plan_phi(pkr_plan* P, double* phi, int phi_on_host)
 
 int64_t pkr_plan_steps(const pkr_plan* P) { return P && P->launches > 0 ? P->launches - 1 : 0; }
 
+int pkr_plan_step_form(pkr_plan* P, int32_t form[5])
+{
+    if (!P || !form) return PKR_EINVAL;
+    int32_t f[3] = {PKR_STEP_SWEEP, P->variant, 0};
+    if (P->stencil && P->form > 0) {
+        f[0] = PKR_STEP_PLANES;
+        f[1] = stencil_cz(P->form);
+        f[2] = stencil_ty(P->form);
+    } else if (P->stencil) {
+        f[0] = PKR_STEP_STENCIL;
+        f[1] = P->form == kStencilParts4 ? 4 : 1;
+    } else if (P->prob.precision == PKR_FP16) {
+        const int h = h16_form(P, P->variant);
+        f[0] = PKR_STEP_SWEEP16;
+        f[1] = h == 2 ? 4 : h == 1 ? 2 : 1;
+        f[2] = h > 0;
+    }
+    for (int k = 0; k < 3; ++k) form[k] = f[k];
+    form[3] = P->grid;
+    form[4] = resident_of(P);
+    return PKR_OK;
+}
+
 void* pkr_plan_populations(pkr_plan* P) { return (P && !P->stencil) ? P->pop[P->cur] : nullptr; }
 
 int pkr_solve(const pkr_problem* p, const double* rho, double* phi, int host_buffers,
