@@ -159,7 +159,10 @@ typedef struct pkr_stats {
                                 ladder): an index into the list pkr_variant_count counts
                                 (pkr_batch_variant_count for a context's request; binary16:
                                 0 one site per lane, 1 several); -1 when no population sweep
-                                ran (scalar stencil, pkr_fixed_point_fft) */
+                                ran (scalar stencil, pkr_fixed_point_fft); -2 when the
+                                population sweep ran in cooperative launches (a
+                                per-step-checked binary64 run on a small grid, see
+                                pkr_plan_run) and not in a geometry of the list */
 } pkr_stats;
 
 /* Human-readable name of a status code (static string). */

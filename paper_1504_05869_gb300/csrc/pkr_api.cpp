@@ -1148,7 +1148,7 @@ int pkr_plan_run(pkr_plan* P, int64_t steps, double tol, int tol_kind, int check
     double min_res = INFINITY;
     int nchecks = 0, since_min = 0;   // checks since the last new minimum
     int64_t done = 0;
-    bool stopped = false;
+    bool stopped = false, resident = false;
     // Binary64 runs that check every step (the per-step stopping rules of
     // small problems): steps go in captured graphs of kGraphSteps, the rule is
     // applied on the device after each check, and the host reads the outcome
@@ -1175,6 +1175,7 @@ int pkr_plan_run(pkr_plan* P, int64_t steps, double tol, int tol_kind, int check
                 PKR_CK(cudaStreamSynchronize(P->stream));
                 const RunCtl c = P->hctl;
                 if (c.status == PKR_ECUDA) return PKR_ECUDA;
+                resident = true;
                 resident_advance(P, form, (int64_t)c.done_at + 1);
                 done += (int64_t)c.done_at + 1;
                 P->last_residual = c.last_res;
@@ -1273,7 +1274,7 @@ int pkr_plan_run(pkr_plan* P, int64_t steps, double tol, int tol_kind, int check
         st->glups = ms > 0 ? upd / (ms * 1e6) : 0.0;
         const double bytes_site = 2.0 * P->lat.Q * P->elem + source_bytes(P->prob.precision);
         st->hbm_gbs = ms > 0 ? upd * bytes_site / (ms * 1e6) : 0.0;
-        st->variant = P->stencil ? -1 : P->variant;
+        st->variant = P->stencil ? -1 : resident ? -2 : P->variant;
     }
     return status;
 }
