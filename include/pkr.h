@@ -205,8 +205,9 @@ int pkr_variant_count(int lattice);
  * unknown lattice. */
 int pkr_batch_variant_count(int lattice);
 
-/* Device bytes a plan for this problem allocates (populations, source, Phi,
- * scratch).  Host only. */
+/* Device bytes a plan for this problem allocates: populations, source, Phi,
+ * scratch, and the third population array that a per-step-checked binary64 run
+ * on a small grid adds (pkr_plan_run).  Host only. */
 int pkr_plan_bytes(const pkr_problem *problem, size_t *bytes);
 
 /* ---------------------------------------------------------------------

@@ -185,7 +185,8 @@ int validate(const pkr_problem* p, LatticeInfo* li, double* tau)
 }  // namespace
 
 // Upper bound on a persistent sweep grid (blocks); sizes the partials scratch.
-constexpr int kMaxGridBlocks = 152 * 32;
+constexpr int kSMs = 152;
+constexpr int kMaxGridBlocks = kSMs * 32;
 
 struct pkr_plan {
     pkr_problem prob;
@@ -449,13 +450,13 @@ static_assert(sizeof(RunCtl) <= 64, "the counter sits at byte 64");
 // Steps per launch of a resident run: tens of milliseconds at most.
 constexpr int64_t kResidentSteps = 8192;
 
-// Tiles of 32 sites per SM up to which the stencil's resident forms take a grid.
-constexpr int kStencilTiles = 4;
+// Tiles of 32 sites per SM up to which the resident forms take a grid.
+constexpr int kStencilTiles = 4, kSweepTiles = 2;
 
 // Form of a resident run of this plan (0: none).  Only where the plan's
 // one-step kernel computes the same values: the per-site stencil, or the
-// library's own choice of sweep geometry.  Tiles: 4 per SM for the stencil,
-// 2 per SM for the sweep (8 + 1 warps of a tile each).
+// library's own choice of sweep geometry.  Tiles: 4 per SM for the stencil, 2
+// per SM for the sweep (a block of up to 15 + 1 warps each).
 int resident_of(pkr_plan* P)
 {
     if (P->resident >= 0) return P->resident;
@@ -463,7 +464,7 @@ int resident_of(pkr_plan* P)
     if (P->prob.precision != PKR_FP64 || P->prob.variant >= 0 ||
         (P->stencil && P->form != kStencilParts4))
         return 0;
-    const int st = P->stencil ? 1 : 0, most = (st ? kStencilTiles : 2) * P->nsm;
+    const int st = P->stencil ? 1 : 0, most = (st ? kStencilTiles : kSweepTiles) * P->nsm;
     switch (P->prob.lattice) {
     case PKR_D1Q5: P->resident = resident_form<D1Q5>(P->V, st, P->nsm, most); break;
     case PKR_D1Q9: P->resident = resident_form<D1Q9>(P->V, st, P->nsm, most); break;
@@ -715,6 +716,11 @@ int pkr_plan_bytes(const pkr_problem* p, size_t* bytes)
     if (!bytes) return PKR_EINVAL;
     const int64_t V = p->n[0] * p->n[1] * p->n[2];
     *bytes = plan_bytes(p, li, V, kMaxGridBlocks);
+    // the third array of resident runs (see resident_of and resident_ready);
+    // tau_lb = 1 steps Phi alone
+    if (p->precision == PKR_FP64 && p->variant < 0 && 1.0 / tau != 1.0 &&
+        (V + 31) / 32 <= kSweepTiles * kSMs)
+        *bytes += (size_t)li.Q * (size_t)V * 8 + 16;
     return PKR_OK;
 }
 
