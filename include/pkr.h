@@ -81,9 +81,9 @@ typedef enum pkr_lattice {
  * arithmetic in binary32, source in binary32; accurate to ~1e-4 of Phi.
  * Where nx is a multiple of 64 and no edge is below the lattice's reach, the
  * sweep gives each lane two adjacent sites, or four where nx is a multiple of
- * 128 and the grid has a 128-site tile for every resident warp (variant 1, the
- * default there; variant 0 keeps one site per lane); all give the same Phi bit
- * for bit between residual checks.
+ * 128 and the grid has enough tiles of 128 sites (8 per SM for D3Q111; see
+ * pkr_plan_step_form) (variant 1, the default there; variant 0 keeps one site
+ * per lane); all give the same Phi bit for bit between residual checks.
  * MIXED16 (pkr_solve only): binary16 to PKR_MIXED16_SWITCH_TOL, binary32 to
  * PKR_MIXED_SWITCH_TOL, then binary64 to tol.
  * A reduced-precision rung also hands over at its rounding floor, which can

@@ -280,12 +280,30 @@ int launch_stencil_step(pkr_plan* P, const double* in, double* out, const double
 }
 
 // binary16: form of the sweep that variant `variant` of this plan runs.
-// Variant 1 takes four sites per lane on x rows of whole 128-site tiles once
-// they give every resident warp (six per SM) a tile, else two.
+// Variant 1 takes four sites per lane on x rows of whole 128-site tiles, from a
+// number of tiles per SM on that its few warps (six per SM of D3Q111, four of
+// D2Q169) share out evenly enough.  Time of a step with four sites per lane to
+// that with two, by tiles of 128 per SM: D3Q111 1.16 (6.1), 1.18 (6.9), 0.98
+// (8.1), 0.89 (8.9), 0.87 (12), 0.85 (26), 0.82 (185); D3Q19 1.02 (6.1), 0.92
+// (12), 0.80 (34), 0.77 (185); D2Q25 0.93 (6.1), 0.97 (8), 0.78 (26), 0.76 (185).
+// Reaches above four need a halo of eight sites, a sixteenth more to copy: D1Q9
+// and D1Q13 1.01 (18), 0.97 (26), 0.78 (92); D2Q81 1.06 (26), 1.01 (53), 0.96
+// (79), 0.92 (158); D2Q169 1.07 (26), 1.06 (53), 1.00 (79), 0.97 (211), but 1.09
+// where every row is one tile.  D1Q5's five planes are too few to gain: 1.06
+// (92), 1.01 (184).
+//   Two sites per lane with copies ahead: D3Q111 only, 0.97 of the time without
+// from 18 tiles of 64 per SM on (1.02 below); D2Q169 1.05, D3Q19 1.01, D2Q81 1.00.
 int h16_form(const pkr_plan* P, int variant)
 {
-    if (variant != 1 || !P->h16pairs) return 0;
-    return P->prob.n[0] % 128 == 0 && P->V / 128 >= (int64_t)6 * P->nsm ? 2 : 1;
+    if (variant != 1 || !P->h16pairs) return kH16One;
+    const int Q = P->lat.Q;
+    const int64_t nx = P->prob.n[0], per_sm = P->V / 128 / P->nsm;
+    const int from = Q < 9 ? 0x7fffffff
+                     : P->lat.reach <= 4 ? (Q <= 64 ? 6 : 8)
+                                         : (Q <= 64 ? 26 : 72);
+    if (nx % 128 == 0 && per_sm >= from && (nx > 128 || Q <= 111)) return kH16Four;
+    return P->prob.lattice == PKR_D3Q111 && P->V / 64 >= (int64_t)18 * P->nsm ? kH16TwoAhead
+                                                                              : kH16Two;
 }
 
 int launch_one(pkr_plan* P, int mode, bool zero_in)
@@ -1311,8 +1329,8 @@ int pkr_plan_step_form(pkr_plan* P, int32_t form[5])
     } else if (P->prob.precision == PKR_FP16) {
         const int h = h16_form(P, P->variant);
         f[0] = PKR_STEP_SWEEP16;
-        f[1] = h == 2 ? 4 : h == 1 ? 2 : 1;
-        f[2] = h > 0;
+        f[1] = h16_sites(h);
+        f[2] = h == kH16TwoAhead || h == kH16Four;
     }
     for (int k = 0; k < 3; ++k) form[k] = f[k];
     form[3] = P->grid;

@@ -41,6 +41,10 @@ enum SweepVariant { kStaged = 0 };
 
 // Storage precision code of binary16 populations (include/pkr.h: PKR_FP16).
 constexpr int kFP16 = 3;
+// Form of a binary16 sweep: sites per lane, and whether a tile's copies start
+// while the one before is relaxed (with four sites they always do).
+enum H16Form { kH16One = 0, kH16Two = 1, kH16TwoAhead = 2, kH16Four = 3 };
+constexpr int h16_sites(int form) { return form == kH16Four ? 4 : form == kH16One ? 1 : 2; }
 // Storage precision code of 64-bit fixed-point populations (PKR_FX64).
 constexpr int kFX64 = 5;
 

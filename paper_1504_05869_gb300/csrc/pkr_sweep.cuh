@@ -1271,7 +1271,9 @@ __device__ __forceinline__ f32x2 h16_pair(uint32_t sw)
     return pack2(v.x, v.y);
 }
 
-template <class L, int TILES, int MINB>
+// AHEAD: a class's slots take the copies of the warp's next tile as soon as it
+// is relaxed.
+template <class L, int TILES, int MINB, bool AHEAD>
 __global__ void __launch_bounds__(TILES * 32, MINB)
 sweep_h16p_kernel(const SweepArgs a, const Coefs<float> c)
 {
@@ -1341,14 +1343,18 @@ sweep_h16p_kernel(const SweepArgs a, const Coefs<float> c)
         }
     };
     const int first = blockIdx.x * TILES + sub;
-    if (first < ntiles) {
+    if (AHEAD && first < ntiles) {
         locate(first);
         static_for<0, Q>(pull);
     }
     for (int tile = first; tile < ntiles; tile += nt) {
+        if constexpr (!AHEAD) {
+            locate(tile);
+            static_for<0, Q>(pull);
+        }
         const int s = tile * 64 + 2 * lane;
         const float2 S2 = *reinterpret_cast<const float2*>(S + s);
-        const bool more = tile + nt < ntiles;
+        const bool more = AHEAD && tile + nt < ntiles;
         if (more) locate(tile + nt);
         cp_async_wait_all();
         __syncwarp();
@@ -1406,9 +1412,12 @@ sweep_h16p_kernel(const SweepArgs a, const Coefs<float> c)
             }
             // the class's slots take the next tile: its copies are in flight
             // while the other classes and the next tile's repack run
-            __syncwarp();
-            if (more) static_for<i0, i1>(pull);
+            if constexpr (AHEAD) {
+                __syncwarp();
+                if (more) static_for<i0, i1>(pull);
+            }
         });
+        if constexpr (!AHEAD) __syncwarp();   // the slots have been read
         if (a.mode != kPlain) {
             const double phA = (double)PhiA, phB = (double)PhiB;
             if (a.mode == kCheck) {
@@ -1476,26 +1485,27 @@ sweep_h16p_kernel(const SweepArgs a, const Coefs<float> c)
 
 namespace pkr {
 
-// binary16 forms: 0 one site per lane (any grid), 1 two sites per lane (nx a
-// multiple of 64 and no edge below the reach; the plan checks), 2 four sites
-// per lane (nx a multiple of 128).  Tiles per block, measured at 256 x 256 x
-// 192, D3Q111: form 1, 2 tiles and 6 blocks per SM 9.90 GLUPS, 7 blocks (128
-// registers) 9.25; form 2, 2 tiles 11.51, 1 tile 10.41, 3 tiles 11.30, 7 tiles
-// 9.93.
+// binary16 forms (H16Form): one site per lane (any grid), two (nx a multiple of
+// 64 and no edge below the reach; the plan checks), two with the next tile's
+// copies in flight, four (nx a multiple of 128).  Tiles per block, measured at
+// 256 x 256 x 192, D3Q111: two sites, copies ahead, 2 tiles and 6 blocks per SM
+// 9.90 GLUPS, 7 blocks (128 registers) 9.25; four sites, 2 tiles 11.51, 1 tile
+// 10.41, 3 tiles 11.30, 7 tiles 9.93.  When the plan takes which: see h16_form.
 constexpr int kH16Tiles = 2;
 template <class L>
 constexpr size_t h16_smem(int form)
 {
-    return form == 2 ? H16w<L>::smem_bytes(kH16Tiles)
-           : form == 1 ? (size_t)kH16Tiles * (L::Q * 33 * 4 + 32 * 4)
-                       : (size_t)kH16Tiles * L::Q * 32 * 4;
+    return form == kH16Four  ? H16w<L>::smem_bytes(kH16Tiles)
+           : form == kH16One ? (size_t)kH16Tiles * L::Q * 32 * 4
+                             : (size_t)kH16Tiles * (L::Q * 33 * 4 + 32 * 4);
 }
 template <class L>
 auto h16_kernel(int form)
 {
-    return form == 2 ? sweep_h16w_kernel<L, kH16Tiles>
-           : form == 1 ? sweep_h16p_kernel<L, kH16Tiles, 6>
-                       : sweep_h16_kernel<L, kH16Tiles>;
+    return form == kH16Four       ? sweep_h16w_kernel<L, kH16Tiles>
+           : form == kH16TwoAhead ? sweep_h16p_kernel<L, kH16Tiles, 6, true>
+           : form == kH16Two      ? sweep_h16p_kernel<L, kH16Tiles, 7, false>
+                                  : sweep_h16_kernel<L, kH16Tiles>;
 }
 
 template <class L>
@@ -1514,7 +1524,7 @@ int occupancy_h16(int form, int* blocks, int* tiles_per_block)
     cudaError_t e = set_sweep_smem(kern, smem);
     if (e != cudaSuccess) return (int)e;
     // tiles_per_block counts 32-site tiles
-    *tiles_per_block = (form == 2 ? 4 : form == 1 ? 2 : 1) * kH16Tiles;
+    *tiles_per_block = h16_sites(form) * kH16Tiles;
     return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kern, kH16Tiles * 32, smem);
 }
 
