@@ -147,11 +147,14 @@ KERNEL_SOURCES = ("pkr_sweep.cuh", "pkr_sweep_pair.cuh", "pkr_sweep_ws.cuh", "pk
                   "sweep_d3q111.cu")
 
 
-def kernel_label(pk, variant):
-    """Name of the sweep kernel a plan variant launches."""
+def kernel_label(pk, variant, form=None):
+    """Name of the sweep kernel a plan variant launches (form: the plan's
+    step_form, which binary16 needs: variant 1 has several forms)."""
     T = {"fp64": "double", "fx64": "long long"}.get(PRECISION, "float")
     if PRECISION == "fp16":
-        return ("sweep_h16p_kernel" if variant == 1 else "sweep_h16_kernel") + f"<{LATTICE}>"
+        lanes, ahead = form[1:3]
+        name = {1: "sweep_h16_kernel", 2: "sweep_h16p_kernel", 4: "sweep_h16w_kernel"}[lanes]
+        return f"{name}<{LATTICE}>" + (" (copies ahead)" if lanes == 2 and ahead else "")
     nb = pk._pkr.pkr_batch_variant_count(pk.LATTICES[LATTICE])   # staged geometries
     nv = pk._pkr.pkr_variant_count(pk.LATTICES[LATTICE])
     if variant < nb:
@@ -162,6 +165,15 @@ def kernel_label(pk, variant):
             return f"sweep_wide_kernel<{LATTICE}>"
         return f"sweep_pair_kernel<{LATTICE},{T},G=2> ({form})"
     return f"sweep_ws_kernel<{LATTICE},{T}>"
+
+
+def stencil_label(form, Q):
+    """Name of the scalar-stencil kernel of a step form, and its binary64
+    operations per site: by planes about 47 (D3Q111) or 13 (D3Q19), else one per
+    velocity, and one more for each of several partial sums."""
+    if form[0] == 3:
+        return f"stencil_planes_kernel<{LATTICE},{form[2]}>", {111: 47, 19: 13}[Q]
+    return f"stencil_kernel<{LATTICE}>", Q if form[1] == 1 else Q + form[1]
 
 
 def kernel_code_hash(texts):
@@ -409,12 +421,12 @@ def run(args):
     prob = pk.problem(LATTICE, SHAPE, ORDER, knudsen=KN, tau_lb=TAU, tol=0.0,
                       check_every=SWEEPS_PER_STEP, max_sweeps=10 ** 9, precision=PRECISION,
                       variant=args.variant)
-    # tau_lb = 1 in binary64 runs the scalar stencil (Phi-only state)
-    stencil = TAU == 1.0 and PRECISION == "fp64"
     r_dev = torch.from_numpy(rho).cuda()
     with torch.cuda.stream(stream):
         plan = pk.Plan(prob, stream=stream)
         plan.load_source(r_dev)
+    # tau_lb = 1 in binary64 runs the scalar stencil (Phi-only state)
+    stencil = plan.step_form()[0] >= pk._pkr.PKR_STEP_STENCIL
     Q = {"D3Q111": 111, "D3Q19": 19}[LATTICE]
     esize = {"fp64": 8, "fx64": 8, "fp32": 4, "fp16": 2}[PRECISION]
     tau = None
@@ -427,6 +439,7 @@ def run(args):
         variant = args.variant
     else:
         variant, tuned_ms = plan.autotune(2)
+    form = plan.step_form()
     for _ in range(args.warmup):
         st = step()
     tau = st["tau_lb"]
@@ -515,22 +528,20 @@ def run(args):
         cpu_full = cpu_full_solve(pk, torch)
 
     if stencil:
-        # binary64 pipe bound: about 47 (D3Q111) or 13 (D3Q19) operations per
-        # site in the plane form that 3D grids of this size run, else Q; peak
-        # from the GB300's nominal FP64 rate (1.25 TFLOP/s = 625 G operations/s)
-        planes = LATTICE in ("D3Q111", "D3Q19") and V >= 1 << 20
-        ops = {"D3Q111": 47, "D3Q19": 13}[LATTICE] if planes else Q
+        # binary64 pipe bound; peak from the GB300's nominal FP64 rate
+        # (1.25 TFLOP/s = 625 G operations/s)
+        kernel, ops = stencil_label(form, Q)
         fma_s = V * ops / (launch_ms * 1e-3) / 1e9
         roofline = {"bound": "alu", "achieved": fma_s, "peak": 625.0, "unit": "GFMA/s",
                     "frac": fma_s / 625.0, "traffic": None, "peak_source": "nominal FP64",
-                    "kernel": f"stencil_{'planes_' if planes else ''}kernel<{LATTICE}>",
+                    "kernel": kernel,
                     "hbm_gbs": achieved,
                     "algorithmic_bytes_per_launch": V * bytes_site}
     else:
         roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak,
                     "unit": "GB/s", "frac": achieved / hbm_peak,
                     "traffic": recorded_traffic(variant), "peak_source": peak_src,
-                    "kernel": kernel_label(pk, variant),
+                    "kernel": kernel_label(pk, variant, form),
                     "algorithmic_bytes_per_launch": V * bytes_site}
     if rank == 0:
         line = {
