@@ -949,9 +949,6 @@ sweep_batch_kernel(BatchState* st, int k, int phase)
             }
             TilePull<L, T> here;
             here.locate(tile - gd.tile_begin, tg.V, tg.nx, tg.ny, tg.nz, tg.small, age == 0, lane);
-            // the next tile's grid is this one or a later one
-            if (tile + nt < ntiles)
-                while (gi + 1 < ngrids && grids[gi + 1].tile_begin <= tile + nt) ++gi;
             double d2 = 0.0, n2 = 0.0, mx = 0.0, ms = 0.0;
             unsigned long long fxm = 0ull;
             groups([&](auto GI) {
@@ -966,6 +963,9 @@ sweep_batch_kernel(BatchState* st, int k, int phase)
                                                 fxm, false, pull);
             });
             finish(gd, tile, mode, d2, n2, mx, ms, fxm);
+            // the next tile's grid is this one or a later one
+            if (tile + nt < ntiles)
+                while (gi + 1 < ngrids && grids[gi + 1].tile_begin <= tile + nt) ++gi;
         }
     };
     // One loop for all groups in binary64, one for each in the other storages,
