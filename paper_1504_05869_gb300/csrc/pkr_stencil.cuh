@@ -19,9 +19,10 @@ namespace pkr {
 // One site from its Q neighbours: the classes fall into kStencilParts
 // contiguous parts of about Q / kStencilParts velocities; part j is
 // sum_c w_c (sum of the class), and the site's value ((a0 + a1) + (a2 + a3)) +
-// St.  Every kernel below but the plane one evaluates exactly this, so they
-// agree bit for bit whether one thread takes all parts or four warps take one
-// each.
+// St.  The resident forms and stencil_kernel with SPLIT evaluate exactly this, so
+// they agree bit for bit whether one thread takes all parts or four warps take
+// one each; stencil_kernel without it (one chain) and the plane form add in
+// orders of their own.
 // ---------------------------------------------------------------------------
 constexpr int kStencilParts = 4;
 
@@ -65,9 +66,6 @@ struct Neighbours {
     static constexpr int WY = L::DIM >= 2 ? W : 1, WZ = L::DIM >= 3 ? W : 1;
     int xs[W], yo[WY], zo[WZ];
 
-    // (signed divisions and one branch on small: with unsigned ones and a choice
-    // per offset the per-site form took 39.9 us a step for 32.9 on 100 x 90 x 80,
-    // D3Q19, in 48 registers for 42)
     __device__ __forceinline__ void locate(int s, int nx, int ny, int nz, int small)
     {
         const int x = s % nx, r = s / nx, y = r % ny, z = r / ny;
@@ -163,10 +161,11 @@ stencil_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t s64 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s64 < V; s64 += stride) {
         const int s = (int)s64;
-        Neighbours<L> nb;
-        nb.locate(s, nx, ny, nz, small);
-        double acc = St ? St[s] : 0.0;
+        double acc;
         if constexpr (SPLIT) {
+            Neighbours<L> nb;
+            nb.locate(s, nx, ny, nz, small);
+            acc = St ? St[s] : 0.0;
             double a[kStencilParts];
             static_for<0, kStencilParts>([&](auto J) {
                 constexpr int j = decltype(J)::value;
@@ -176,9 +175,30 @@ stencil_kernel(const double* __restrict__ Pin, double* __restrict__ Pout,
             });
             acc = ((a[0] + a[1]) + (a[2] + a[3])) + acc;
         } else {
+            // (offsets on three axes for every set, and a choice per offset: as
+            // Neighbours forms them D2Q81 took 9.0 us a step for 8.3 on 150 x 150,
+            // the other sets the same within 1 %)
+            constexpr int RC = reach_of<L>(), W = 2 * RC + 1;
+            const int nxy = nx * ny;
+            const int x = s % nx, r = s / nx, y = r % ny, z = r / ny;
+            int xs[W], yo[W], zo[W];
+#pragma unroll
+            for (int d = -RC; d <= RC; ++d) {
+                if (small) {
+                    xs[d + RC] = wrap_any(x - d, nx);
+                    yo[d + RC] = wrap_any(y - d, ny) * nx;
+                    zo[d + RC] = wrap_any(z - d, nz) * nxy;
+                } else {
+                    xs[d + RC] = wrap_near(x - d, nx);
+                    yo[d + RC] = wrap_near(y - d, ny) * nx;
+                    zo[d + RC] = wrap_near(z - d, nz) * nxy;
+                }
+            }
+            acc = St ? St[s] : 0.0;
             static_for<0, L::Q>([&](auto I) {
                 constexpr int i = decltype(I)::value;
-                acc = fma(c.wphi[cls_of<L>(i)], __ldg(Pin + nb.template at<i>()), acc);
+                const int at = zo[vz_of<L>(i) + RC] + yo[vy_of<L>(i) + RC] + xs[vx_of<L>(i) + RC];
+                acc = fma(c.wphi[cls_of<L>(i)], __ldg(Pin + at), acc);
             });
         }
         Pout[s] = acc;
