@@ -15,8 +15,8 @@
 // out behind the steps, off their critical path: a step or two later a warp
 // that takes no part in the stencil decides, and the step's result is still
 // there (in a third buffer, or in registers).  Whole solves, before and now:
-// 64-site D1Q13 line at tau_lb = 1, 4200 steps, 38.8 -> 3.4 ms (5.9 with one
-// checking warp); 64^2 D2Q169 at Kn 0.1, 208 steps, 4.6 -> 2.1 ms.
+// 64-site D1Q13 line at tau_lb = 1, 4200 steps, 39.2 -> 3.05 ms (5.9 with one
+// checking warp); 64^2 D2Q169 at Kn 0.1, 208 steps, 4.6 -> 1.7 ms.
 #pragma once
 
 namespace pkr {

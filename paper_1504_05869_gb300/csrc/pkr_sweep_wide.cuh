@@ -23,8 +23,9 @@ struct Wide {
     static constexpr int HL = (reach_of<L>() + 3) / 4 * 4;   // halo values per side
     static constexpr int RL = 64 + 2 * HL;
     static constexpr int ROWB = RL * 4;
-    // 64-site pairs per block: one block of 12 warps per SM.  GB/s at 192^3 and
-    // 256 x 256 x 160, D3Q111: 6 pairs 5905 / 5807, 4 pairs 5898 / 5748 (8
+    // 64-site pairs per block: one block of 12 warps per SM.  Measured on D3Q111
+    // (D2Q81 takes the same; D2Q169's rows leave room for 3).  GB/s at 192^3 and
+    // 256 x 256 x 160: 6 pairs 5905 / 5807, 4 pairs 5898 / 5748 (8
     // warps), 3 pairs x 2 blocks 5713 / 5697, 2 pairs x 3 blocks 4877 / 4875,
     // 7 pairs 4631 / 4570 (too little of the SM left for L1).
     static constexpr int PAIRS = L::Q > 111 ? 3 : 6;
